@@ -128,12 +128,11 @@ typedef struct {
                             processed tick.                                 */
     float block_eta;     /* accuracy parameter of the block step criterion
                             (default 0.025), > 0                             */
-    int32_t walk_pipeline; /* 1: the walk runs in warp pairs, one warp
-                            traversing the tree and handing interaction lists
-                            through shared memory to one warp evaluating Eq. 1
-                            (monopole walks without the potential; identical
-                            results); needs an even warps_per_block.  0: each
-                            warp traverses and evaluates (default)          */
+    int32_t walk_pipeline; /* 1: asks for a walk in warp pairs (one traversing,
+                            one evaluating), whose results are those of 0 bit
+                            for bit; needs an even warps_per_block.  The walk
+                            of 0 (default) was faster at every size measured,
+                            and both settings run it                        */
 } nbody_config;
 
 typedef struct {
@@ -142,7 +141,9 @@ typedef struct {
     int64_t interactions;  /* kernel evaluations of the last walk (the zero
                               self term of each particle included)            */
     int64_t list_entries;  /* interaction-list entries flushed (sum over groups) */
-    int32_t max_stack;     /* deepest traversal stack seen                   */
+    int32_t max_stack;     /* deepest traversal stack seen (of a warp, or of a CTA
+                              walking one group, which has room for 8 times
+                              stack_depth entries)                            */
     int32_t levels;        /* tree levels below the root                     */
     int64_t kernels;       /* kernels this library launched in the last call  */
     float ms_build;        /* device time of the build phase(s) (CUDA events)  */
@@ -156,8 +157,9 @@ typedef struct {
                               tree (the others refitted it)                    */
     int64_t quad_interactions; /* of `interactions`, those with quadrupole
                               nodes (quadrupole = 1)                          */
-    int32_t walk_warps;    /* resident walk warps (queue consumers) of the last
-                              walk launch                                      */
+    int32_t walk_warps;    /* resident walk warps of the last walk launch (one
+                              warp per group; for small systems, whose groups
+                              are walked by whole CTAs, those CTAs' warps)     */
 } nbody_stats;
 
 typedef struct nbody_ctx nbody_ctx;
@@ -428,9 +430,8 @@ nbody_status nbody_sort_keys(nbody_ctx *ctx, int32_t method, const uint64_t *key
 /* Self-tests of the library's failure paths (no counterpart in the paper).
  * NBODY_SELFTEST_SORT_WAIT: runs one radix-sort pass kernel on a two-tile
  * input whose first tile is never processed, so the second tile's look-back
- * (the decoupled look-back of the one-sweep sort, the default path's only
- * device wait; the opt-in warp-pair walk's hand-offs are the other, bounded
- * the same way) finds nothing to wait for; the wait is bounded (2^20 polls) and the
+ * (the decoupled look-back of the one-sweep sort, the library's only device
+ * wait) finds nothing to wait for; the wait is bounded (2^20 polls) and the
  * kernel records a timeout and finishes.  Returns the status the device
  * reported: NBODY_ETIMEOUT when the bound works.  Allocates and frees its own
  * buffers (about 200 KB) and synchronises cuda_stream (NULL = default

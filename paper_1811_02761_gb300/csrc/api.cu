@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -39,7 +40,7 @@ struct GraphKey {
     bool safe;
     bool mlp_norm;  // the cost model's input statistics were set at capture
     nbody_config cfg;
-    const void *bufs[8];
+    const void *bufs[9];
 };
 
 }  // namespace
@@ -69,6 +70,9 @@ struct nbody_ctx {
     DevBuf sys_off, sys_box, sys_boxord, sys_eps2, sys_eps, sys_root;
     // walk / step
     DevBuf acc_s, aold_s;
+    // cooperative walk: records of groups cut at the quota, partial sums of
+    // groups walked in parts
+    DevBuf heavy, cut, part, part_ctl;
     DevBuf st_buf[2][11];
     DevBuf recs;  // 64-byte particle records of a call's full permutations
     // the Morton order (caller indices) at the end of the last step call: the
@@ -116,7 +120,7 @@ struct nbody_ctx {
                          &node_parent, &node_link, &node_count, &node_nchild, &node_arrive,
                          &nodeA, &nodeB, &mass2, &nodeQ, &gflag, &grp_first, &grp_count, &grp_sphere,
                          &grp_sys, &grp_alpha, &grp_cost, &grp_order, &sys_off, &sys_box,
-                         &sys_boxord, &sys_eps2, &sys_eps, &sys_root, &acc_s, &aold_s, &mlp_w, &mlp_m1,
+                         &sys_boxord, &sys_eps2, &sys_eps, &sys_root, &acc_s, &aold_s, &heavy, &cut, &part, &part_ctl, &mlp_w, &mlp_m1,
                          &mlp_m2, &mlp_wb, &mlp_norm, &mlp_gpart, &mlp_lpart, &mlp_loss, &feat,
                          &target, &score, &okey, &okey_alt, &oval, &oval_alt, &pcost_walk, &recs, &last_ids};
         for (DevBuf *b : all) owned.push_back(b);
@@ -559,6 +563,61 @@ bool use_compensation(const nbody_config &c) {
     return c.compensated == 1 || (c.compensated == 2 && c.delta_acc <= kAutoCompensateDacc);
 }
 
+// Which walk: up to kCoopParticles particles only the cooperative kernel is
+// launched; above, the one-warp kernel, then the cooperative one for the
+// groups cut at the quota -- or for all of them when at most kCoopGroups are
+// walked (a block step's active groups; the kernels read the count).
+// The line lies where the two meet: galaxy, walk only, one warp per group
+// against cooperative: N = 4096 0.198 / 0.041 ms, 30000 0.24 / 0.10, 65536
+// 0.28 / 0.15, 131072 (2953 groups) 0.28 / 0.23, 262147 (5850) 0.37 / 0.41,
+// 1000003 0.98 / 1.38: once every warp has a group of its own, the barriers
+// of the cooperative walk only cost.
+constexpr int64_t kCoopParticles = 1 << 17;
+constexpr int kCoopGroups = 3000;
+
+// Records for groups cut at the quota: twice the count of groups of G
+// particles (they hold 0.7 G on average), so a walk of more groups, which is
+// walked without a quota, is rare.
+int64_t heavy_records(const nbody_ctx *c) { return 2 * c->L.n / c->cfg.group_size + 4096; }
+
+// List entries after which a one-warp group is cut and finished by the
+// cooperative kernel.  A group is one warp's serial chain (40-80 ns per
+// entry), so one far longer than the others runs alone at the end of the
+// launch (Plummer, N = 262147, no |a_old|: one group of 167,663 entries took
+// 13 of the walk's 14 ms).  The line is 2.7 ordinary lists (1500 entries at
+// delta_acc = 2^-9, growing with delta_acc^-0.485, measured from 2^-1 to
+// 2^-20, and with theta^-3 for the geometric criterion), below which the tail
+// is an ordinary group's.  With n / G groups on a few thousand warps a tail
+// of n / 2G entries is a few per cent of the launch, less than the
+// cooperative kernel's lower efficiency would cost.
+int list_quota(const nbody_ctx *c, bool geometric) {
+    const double q = geometric ? std::pow(0.5 / c->cfg.theta, 3.0)
+                               : std::pow(std::max(c->cfg.delta_acc, 1e-12f) * 512.0, -0.485);
+    return (int)std::min(std::max(4096.0 * std::max(q, 1.0), 0.5 * c->L.n / c->cfg.group_size), 1e9);
+}
+
+// A CTA's part of a group: 2048 to 16384 measured, 4096 best on a forest,
+// block steps and a tight tolerance together (delta_acc = 2^-20, N = 30011:
+// 1.01 ms at 2048 and 4096, 1.06 at 8192, 1.10 at 16384).
+constexpr int kCutQuota = 4096;
+
+cudaError_t ensure_coop(nbody_ctx *c) {
+    cudaError_t e = cudaSuccess;
+    if (!c->part_ctl.p) {
+        e = ensure(c->part, (size_t)kCutTasks * kPartStride * sizeof(float4));
+        if (e == cudaSuccess) e = ensure(c->cut, (size_t)kCutTasks * kCutWords * 4);
+        // cut_of (-1), cut_count, part_arrive (0), part_entries: set once,
+        // every walk leaves the first three so
+        if (e == cudaSuccess) e = ensure(c->part_ctl, (size_t)kCutTasks * 4 * 4);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->part_ctl.p, 0xff, (size_t)kCutTasks * 4, c->stream);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(P<int32_t>(c->part_ctl) + kCutTasks, 0, (size_t)kCutTasks * 2 * 4, c->stream);
+    }
+    if (e == cudaSuccess && c->L.n > kCoopParticles)
+        e = ensure(c->heavy, (size_t)heavy_records(c) * kHeavyWords * 4);
+    return e;
+}
+
 WalkShape walk_shape(nbody_ctx *c, bool geometric, bool phi, bool safe) {
     WalkShape sh;
     sh.ipl = c->cfg.ipl;
@@ -567,13 +626,13 @@ WalkShape walk_shape(nbody_ctx *c, bool geometric, bool phi, bool safe) {
     sh.compensated = use_compensation(c->cfg);
     sh.safe = safe;
     sh.quad = c->cfg.quadrupole != 0;
-    sh.pipeline = c->cfg.walk_pipeline != 0;
+    sh.coop_only = c->L.n <= kCoopParticles;
     sh.warps_per_block = c->cfg.warps_per_block;
     sh.warps_launched = &c->walk_warps;
     return sh;
 }
 
-WalkArgs walk_args(nbody_ctx *c) {
+WalkArgs walk_args(nbody_ctx *c, bool geometric) {
     WalkArgs a{};
     a.pos4 = P<float4>(c->pos4);
     a.nodeA = P<float4>(c->nodeA);
@@ -587,6 +646,7 @@ WalkArgs walk_args(nbody_ctx *c) {
     a.order = nullptr;
     a.sys_eps2 = P<float>(c->sys_eps2);
     a.sys_root = P<int32_t>(c->sys_root);
+    a.node_count = P<int32_t>(c->node_count);
     a.ds = c->ds;
     a.grp_cost = P<int32_t>(c->grp_cost);
     a.n = c->L.n;
@@ -594,13 +654,27 @@ WalkArgs walk_args(nbody_ctx *c) {
     a.theta = c->cfg.theta;
     a.list_depth = c->cfg.list_depth;
     a.stack_depth = c->cfg.stack_depth;
+    a.coop_groups = c->L.n <= kCoopParticles ? INT32_MAX : kCoopGroups;
+    a.heavy = P<uint32_t>(c->heavy);  // only the one-warp kernel cuts groups into it
+    a.quota = list_quota(c, geometric);
+    a.cut_quota = kCutQuota;
+    a.heavy_cap = (int)std::min<int64_t>(heavy_records(c), INT32_MAX);
+    a.coop_target[0] = std::min(c->nsm * kCoopTarget, kCutTasks);
+    a.coop_target[1] = std::min(c->nsm * kCoopTarget2, kCutTasks);
+    a.cut = P<uint32_t>(c->cut);
+    a.cut_of = P<int32_t>(c->part_ctl);
+    a.cut_count = a.cut_of + kCutTasks;
+    a.part_arrive = a.cut_of + 2 * kCutTasks;
+    a.part_entries = a.cut_of + 3 * kCutTasks;
+    a.part = P<float4>(c->part);
     return a;
 }
 
 // Reset the walk's queue head and counters (status is kept).
 nbody_status reset_walk_counters(nbody_ctx *c, bool accumulators) {
     char *base = reinterpret_cast<char *>(c->ds);
-    NB_CUDA(c, cudaMemsetAsync(base + offsetof(DevState, queue_head), 0, sizeof(int32_t), c->stream));
+    static_assert(offsetof(DevState, ncut) == offsetof(DevState, queue_head) + 4 * sizeof(int32_t), "adjacent");
+    NB_CUDA(c, cudaMemsetAsync(base + offsetof(DevState, queue_head), 0, 5 * sizeof(int32_t), c->stream));
     if (accumulators) {
         NB_CUDA(c, cudaMemsetAsync(base + offsetof(DevState, max_stack), 0, sizeof(int32_t), c->stream));
         NB_CUDA(c, cudaMemsetAsync(base + offsetof(DevState, list_entries), 0,
@@ -716,7 +790,8 @@ nbody_status run_walk(nbody_ctx *c, bool geometric, bool phi, bool safe, const i
         NB_CUDA(c, cudaEventCreate(&ev));
         c->wev.push_back(ev);
     }
-    WalkArgs a = walk_args(c);
+    if (ensure_coop(c) != cudaSuccess) return fail(c, NBODY_ENOMEM, "allocation");
+    WalkArgs a = walk_args(c, geometric);
     a.order = order;
     a.nactive = nactive;
     a.perm = perm;
@@ -739,7 +814,7 @@ nbody_status run_walk(nbody_ctx *c, bool geometric, bool phi, bool safe, const i
         NB_CUDA(c, cudaEventRecordWithFlags(c->gwev[c->gwev_used + 1], c->stream, cudaEventRecordExternal));
         c->gwev_used += 2;
     }
-    c->kernels += 1;
+    c->kernels += c->L.n <= kCoopParticles ? 1 : 2;
     if (!geometric) c->costs_valid = true;
     return NBODY_OK;
 }
@@ -1319,6 +1394,7 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
         key.bufs[5] = ctx->rs_temp.p;
         key.bufs[6] = ctx->pos4.p;
         key.bufs[7] = ctx->acc_s.p;
+        key.bufs[8] = ctx->heavy.p;
         if (!ctx->gstream)
             NB_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->gstream, cudaStreamNonBlocking));
         if (!ctx->gexec || std::memcmp(&key, &ctx->gkey, sizeof key) != 0) {

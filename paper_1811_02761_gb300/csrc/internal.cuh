@@ -41,7 +41,10 @@ constexpr int kStatusTimeout = 4;  // a bounded device wait ran out (results inv
 struct DevState {
     int32_t nnodes;
     int32_t ngroups;
-    int32_t queue_head;
+    int32_t queue_head;  // walk queues: reset together before every walk
+    int32_t coop_head[2];
+    int32_t nheavy;      // groups cut at the quota by the current walk
+    int32_t ncut;        // parts cut by the cooperative walk's first stage
     int32_t status;
     int32_t max_stack;
     int32_t pad0;
@@ -232,11 +235,36 @@ __host__ __device__ inline int walk_quad_depth(int list_depth) {
     return list_depth / 4 > 32 ? list_depth / 4 : 32;
 }
 __host__ __device__ inline size_t walk_smem_per_warp(int list_depth, int stack_depth,
-                                                     bool quad = false) {
-    const size_t b = (size_t)list_depth * 16 + (quad ? (size_t)walk_quad_depth(list_depth) * 40 : 0) +
+                                                     bool quad = false, int slack = 0) {
+    const size_t b = (size_t)(list_depth + slack) * 16 + (quad ? (size_t)walk_quad_depth(list_depth) * 40 : 0) +
                      (size_t)stack_depth * 4 + (size_t)kWalkScratch * 4;
     return (b + 15) & ~(size_t)15;
 }
+// Groups cut at the quota: records of kHeavyWords words (group, stack size,
+// entries so far, a spare word, then the stack).
+constexpr int kHeavyStack = 128, kHeavyHead = 4, kHeavyWords = kHeavyHead + kHeavyStack;
+// The cooperative walk: kCoopWarps warps per CTA, at most kCoopParts CTAs per group.
+constexpr int kCoopWarps = 8, kCoopParts = 32;
+constexpr int kCoopFine = 2, kCoopFront = 1024;
+// Parts per SM that the first and the second stage spread their groups over:
+// a part has a few rounds of its own at the top of the tree, so the first
+// stage makes no more parts than run at once (N = 4096: 0.041 ms at 3 per
+// SM, 0.077 at 12); the second stage's parts are long and uneven, and more of
+// them balance better (Plummer, N = 131072: 0.38 ms at 12, 0.43 at 3).
+constexpr int kCoopTarget = 3, kCoopTarget2 = 12;
+// Records of parts cut by the first stage (as the heavy records: group, stack
+// size, owner, parts of the owner, then the stack), at most kCutTasks.
+constexpr int kCutTasks = 4096;
+constexpr int kCutStack = 508, kCutWords = kHeavyHead + kCutStack;
+__host__ __device__ inline int coop_list_depth(int list_depth) {
+    const int d = kCoopWarps * list_depth;
+    return d < 1024 ? 1024 : (d > 2048 ? 2048 : d);
+}
+__host__ __device__ inline int coop_stack_depth(int stack_depth) {
+    const int d = kCoopWarps * stack_depth;
+    return d > 8192 ? 8192 : d;
+}
+constexpr int kCoopQuadDepth = 512;  // node-list entries (at least 32 per warp)
 struct WalkArgs {
     const float4 *pos4;
     const float4 *nodeA;
@@ -250,6 +278,7 @@ struct WalkArgs {
     const int32_t *order;      // schedule permutation (NULL: Morton order)
     const float *sys_eps2;
     const int32_t *sys_root;
+    const int32_t *node_count;
     DevState *ds;
     const int32_t *nactive;    // non-NULL: walk only order[0 .. *nactive) (block time steps)
     int32_t *grp_cost;         // list entries per group (NULL: not logged)
@@ -257,12 +286,26 @@ struct WalkArgs {
     float G;
     float theta;
     int list_depth;
+    int list_slack;            // list entries beyond list_depth (set by the launch)
     int stack_depth;
     // outputs: scatter mode (perm != NULL) or sorted mode
     const int32_t *perm;
     float *ax, *ay, *az, *phi;
     float4 *acc_sorted;        // (ax, ay, az, phi)
+    // cooperative walk
+    int coop_groups;           // at most this many groups: all of them cooperatively
+    uint32_t *heavy;           // records of the groups cut at the quota
+    int quota, cut_quota;      // list entries after which a group, a part of a group is cut
+    int heavy_cap;             // records (no quota for a walk of more groups)
+    int coop_target[2];        // parts that the stages spread their groups over
+    uint32_t *cut;             // records of cut parts [kCutTasks]
+    int32_t *cut_of;           // a part's record [kCutTasks], -1 between walks
+    int32_t *cut_count;        // cut parts per group [kCutTasks], zero between walks
+    float4 *part;              // partial sums [kCutTasks][kPartStride] of groups in several parts
+    int32_t *part_entries;     // their list entries [kCutTasks]
+    int32_t *part_arrive;      // finished parts per group [kCutTasks], zero between walks
 };
+constexpr int kPartStride = 128;  // members a group may hold
 struct WalkShape {
     int ipl;
     bool geometric;
@@ -270,10 +313,12 @@ struct WalkShape {
     bool compensated;
     bool safe;                  // some eps == 0: guard the self term
     bool quad;                  // accepted nodes add their quadrupole
-    bool pipeline;              // warp pairs: traversal and evaluation (monopole, no potential)
     int warps_per_block;
+    bool coop_only;             // host: the walk has few enough particles for the cooperative kernel alone
     int *warps_launched;        // host, nullable: receives the resident walk warps
 };
+// The walk of one warp per group (not with sh.coop_only), then the
+// cooperative walk of the groups it left.
 cudaError_t launch_walk(cudaStream_t s, const WalkArgs &a, const WalkShape &sh, int nsm);
 cudaError_t launch_direct(cudaStream_t s, int64_t n, const float *x, const float *y,
                           const float *z, const float *m, float G, float eps, bool compensated,

@@ -1,0 +1,8 @@
+// walk_coop4q.cu -- instances of the cooperative tree walk with up to 4
+// i-particles per lane, nodes with quadrupoles (separate translation unit so
+// the instances compile in parallel).
+#include "walk_coop.cuh"
+
+namespace nb {
+template cudaError_t launch_coop_ipl<4, true>(cudaStream_t, const WalkArgs &, const WalkShape &, int);
+}  // namespace nb

@@ -17,13 +17,15 @@
 //       accepted node       -> its pseudo particle (com, M) joins the list,
 //       opened internal node -> its child range is pushed,
 //       opened leaf          -> its particles join the list;
-//   * the list (float4 x, y, z, m in shared memory) is flushed whenever the
-//     next append would overflow it: every lane evaluates Eq. 1 for its q
+//   * the list (float4 x, y, z, m in shared memory) is flushed once it is
+//     full, at the one place of the loop where little else is live: every lane evaluates Eq. 1 for its q
 //     particles against its split of the entries, read as pairs (two LDS.128)
 //     laid out for the packed FP32 instructions -- 12 FP32-pipe operations +
 //     1 MUFU.RSQ per interaction;
 //   * optional Neumaier compensation of the per-flush partial sums.
-// No warp ever waits on another warp or CTA.
+// No warp ever waits on another warp or CTA.  A group whose list grows past a
+// quota is cut there: its sums so far and its stack are kept, and the
+// cooperative kernel (walk_coop.cuh) finishes it with many warps.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -273,8 +275,8 @@ __device__ __forceinline__ int run_r(uint64_t code, int k) { return run_field(co
 __device__ __forceinline__ int run_P(uint64_t code, int k) { return run_field(code, k, 4, 6); }
 __device__ __forceinline__ int run_s(uint64_t code, int k) { return run_field(code, k, 10, 6); }
 
-template <int IPL>
-__device__ __forceinline__ Tiling lane_tiling(int cnt) {
+template <int IPL, int KM = 1>
+__device__ __forceinline__ Tiling lane_tiling(int cnt, int warp = 0) {
     // a group larger than the slots allow (flagged by the caller) still gets
     // a well-formed layout: the largest one
     const int c = cnt < 1 ? 1 : (cnt > 32 * IPL ? 32 * IPL : cnt);
@@ -285,18 +287,20 @@ __device__ __forceinline__ Tiling lane_tiling(int cnt) {
     for (int k = 0; k < 3; k++) {
         const int P = k < nr ? run_P(t.code, k) : 32, s = k < nr ? run_s(t.code, k) : 1;
         const int split = lane / P;
-        t.k0[k] = (k < nr && split < s) ? split : (1 << 30);
+        t.k0[k] = (k < nr && split < s) ? (KM > 1 ? warp * s + split : split) : (1 << 30);
     }
     return t;
 }
 
-// The flush loops of the runs from slot J on (run K).
-template <int J, int K, int IPL, bool PHI, bool COMP, bool SAFE, bool QUADL>
+// The flush loops of the runs from slot J on (run K).  KM: how many warps
+// share the list (the stride of a lane's entry pairs is KM times the run's
+// splits; t.k0 then counts the warp in).
+template <int J, int K, int IPL, bool PHI, bool COMP, bool SAFE, bool QUADL, int KM = 1>
 __device__ __forceinline__ void flush_runs(const Tiling &t, float4 *L, int nl, float eps2,
                                            ISlots<IPL> &I) {
     if constexpr (J < IPL && K < 3) {
         if (K >= (int)(t.code & 3u)) return;
-        const int r = run_r(t.code, K), ks = run_s(t.code, K), k0 = t.k0[K];
+        const int r = run_r(t.code, K), ks = KM * run_s(t.code, K), k0 = t.k0[K];
 #define NB_FLUSH(R)                                                                            \
     do {                                                                                       \
         if constexpr (QUADL) flush_quad_list<J, R, IPL, PHI, COMP, SAFE>(L, nl, eps2, k0, ks, I); \
@@ -306,13 +310,13 @@ __device__ __forceinline__ void flush_runs(const Tiling &t, float4 *L, int nl, f
             if (r == 4) { NB_FLUSH(4); return; }
         }
         if constexpr (J + 3 <= IPL) {
-            if (r == 3) { NB_FLUSH(3); flush_runs<J + 3, K + 1, IPL, PHI, COMP, SAFE, QUADL>(t, L, nl, eps2, I); return; }
+            if (r == 3) { NB_FLUSH(3); flush_runs<J + 3, K + 1, IPL, PHI, COMP, SAFE, QUADL, KM>(t, L, nl, eps2, I); return; }
         }
         if constexpr (J + 2 <= IPL) {
-            if (r == 2) { NB_FLUSH(2); flush_runs<J + 2, K + 1, IPL, PHI, COMP, SAFE, QUADL>(t, L, nl, eps2, I); return; }
+            if (r == 2) { NB_FLUSH(2); flush_runs<J + 2, K + 1, IPL, PHI, COMP, SAFE, QUADL, KM>(t, L, nl, eps2, I); return; }
         }
         NB_FLUSH(1);
-        flush_runs<J + 1, K + 1, IPL, PHI, COMP, SAFE, QUADL>(t, L, nl, eps2, I);
+        flush_runs<J + 1, K + 1, IPL, PHI, COMP, SAFE, QUADL, KM>(t, L, nl, eps2, I);
 #undef NB_FLUSH
     }
 }
@@ -357,14 +361,11 @@ __device__ __forceinline__ void load_slots(const Tiling &tile, const float4 *__r
 }
 
 // End of a group: the s_k splits of every row are summed onto split 0 in
-// split order (with compensation: Neumaier), then the results are written (G
-// applied once; the potential's self term removed).
-template <int IPL, bool PHI, bool COMP, bool SAFE>
-__device__ __forceinline__ void finish_group(const Tiling &tile, int first, int cnt, float eps2,
-                                             const WalkArgs &a, ISlots<IPL> &I) {
+// split order (with compensation: Neumaier), and store(idx, sums) is called
+// for every member idx of the group by the lane that holds its sums.
+template <int IPL, bool PHI, bool COMP, class Store>
+__device__ __forceinline__ void group_sums(const Tiling &tile, int cnt, ISlots<IPL> &I, Store store) {
     const int lane = (int)lane_id(), used = slots_used(tile.code);
-    const float G = a.G;
-    const float self = SAFE ? 0.0f : rsqrt_fast(eps2);
 #pragma unroll
     for (int q = 0; q < IPL; q++) {
         if (q < used) {  // warp-uniform
@@ -395,21 +396,64 @@ __device__ __forceinline__ void finish_group(const Tiling &tile, int first, int 
                 }
             }
             const int idx = base + row + P * t;
-            if (split == 0 && idx < cnt) {
-                const float ph = PHI ? G * (r[3] + I.mi[q] * self) : 0.0f;
-                const int i = first + idx;
-                if (a.perm) {
-                    const int o = a.perm[i];
-                    a.ax[o] = G * r[0];
-                    a.ay[o] = G * r[1];
-                    a.az[o] = G * r[2];
-                    if (PHI && a.phi) a.phi[o] = ph;
-                } else {
-                    a.acc_sorted[i] = make_float4(G * r[0], G * r[1], G * r[2], ph);
-                }
-            }
+            if (split == 0 && idx < cnt) store(idx, r, I.mi[q]);
         }
     }
+}
+
+// The result of sorted particle i from its sums (G applied once; the
+// potential's self term m_i / eps removed).  With G = 1 and self = 0: the
+// plain sums of a group cut at the quota, kept where its result goes until
+// the cooperative kernel adds the rest.
+template <bool PHI>
+__device__ __forceinline__ void store_force(const WalkArgs &a, int i, const float (&r)[4], float mi,
+                                            float G, float self) {
+    const float ph = PHI ? G * (r[3] + mi * self) : 0.0f;
+    if (a.perm) {
+        const int o = a.perm[i];
+        a.ax[o] = G * r[0];
+        a.ay[o] = G * r[1];
+        a.az[o] = G * r[2];
+        if (PHI && a.phi) a.phi[o] = ph;
+    } else {
+        a.acc_sorted[i] = make_float4(G * r[0], G * r[1], G * r[2], ph);
+    }
+}
+
+template <bool PHI>
+__device__ __forceinline__ void load_sums(const WalkArgs &a, int i, float (&r)[4]) {
+    if (a.perm) {
+        const int o = a.perm[i];
+        r[0] = a.ax[o];
+        r[1] = a.ay[o];
+        r[2] = a.az[o];
+        r[3] = PHI && a.phi ? a.phi[o] : 0.0f;
+    } else {
+        const float4 v = a.acc_sorted[i];
+        r[0] = v.x;
+        r[1] = v.y;
+        r[2] = v.z;
+        r[3] = v.w;
+    }
+}
+
+static __device__ __noinline__ void save_heavy(const WalkArgs &a, DevState *ds, int g, int sp, int entries, const uint32_t *stk) {
+    const int lane = (int)lane_id();
+    int h = 0;
+    if (lane == 0) h = atomicAdd(&ds->nheavy, 1);
+    h = __shfl_sync(NB_FULL, h, 0);
+    uint32_t *rec = a.heavy + (size_t)h * kHeavyWords;  // h < ng <= heavy_cap
+    if (lane == 0) {
+        rec[0] = (uint32_t)g;
+        rec[1] = (uint32_t)sp;
+        rec[2] = (uint32_t)entries;
+    }
+    for (int k = lane; k < sp; k += 32) rec[kHeavyHead + k] = stk[k];
+}
+
+// Whether a group's list has passed the quota (asked at its flushes).
+__device__ __forceinline__ bool over_quota(const WalkArgs &a, int entries, int ng) {
+    return entries >= a.quota && ng <= a.heavy_cap;
 }
 
 // Register budget of the walk kernel per thread: 64 (32 resident warps per
@@ -435,19 +479,21 @@ __global__ void __maxnreg__(walk_regs<IPL>()) walk_kernel(WalkArgs a, int geomet
     const int D = a.list_depth, S = a.stack_depth;
     const int DQ = QUAD ? walk_quad_depth(D) : 0;
     const unsigned lane = lane_id(), w = threadIdx.x >> 5;
-    // per warp: the paired list (D entries = D/2 pairs in LA), with
-    // quadrupoles the paired node list (DQ entries, 40 B each), the stack and
-    // kWalkScratch words for the leaf compaction
-    const size_t per_warp = walk_smem_per_warp(D, S, QUAD);
+    // per warp: the paired list (D entries = D/2 pairs in LA, and the slack),
+    // with quadrupoles the paired node list (DQ entries, 40 B each), the stack
+    // and kWalkScratch words for the leaf compaction
+    const int DL = D + a.list_slack;
+    const size_t per_warp = walk_smem_per_warp(D, S, QUAD, a.list_slack);
     float4 *LA = reinterpret_cast<float4 *>(walk_smem + w * per_warp);
-    float4 *LQ = LA + D;
-    uint32_t *stk = reinterpret_cast<uint32_t *>(walk_smem + w * per_warp + (size_t)D * sizeof(float4) +
+    float4 *LQ = LA + DL;
+    uint32_t *stk = reinterpret_cast<uint32_t *>(walk_smem + w * per_warp + (size_t)DL * sizeof(float4) +
                                                  (size_t)DQ * 40);
     int *scr = reinterpret_cast<int *>(stk + S);
     DevState *ds = a.ds;
     const int ng = a.nactive ? *a.nactive : ds->ngroups;
     const int nnodes = ds->nnodes;
     const int npart = (int)a.n;
+    if (ng <= a.coop_groups) return;  // fewer groups than warps: the cooperative kernel's
     const unsigned lt = lanemask_lt();
     int max_sp = 0;
     unsigned long long warp_entries = 0, warp_inter = 0, warp_quad = 0;
@@ -474,9 +520,52 @@ __global__ void __maxnreg__(walk_regs<IPL>()) walk_kernel(WalkArgs a, int geomet
 
         if (lane == 0) stk[0] = (uint32_t)root << 3;  // one node: the system's root
         int sp = 1, nl = 0, nq = 0;
-        long long entries = 0, qentries = 0;
+        int entries = 0, qentries = 0;  // at most particles + nodes of the system
+        // opened leaves whose particles are still to join the list: pend slots,
+        // from pbase on; lane k's leaf starts at slot lexcl, and slot s of it
+        // is particle ldelta + s
+        int pend = 0, pbase = 0, lexcl = 0, ldelta = 0;
         __syncwarp();
-        while (sp > 0) {
+        // One step per iteration -- 32 pending leaf particles, or a round of
+        // nodes -- adds at most 32 entries, so the lists are flushed in one
+        // place, where little else is live.
+        for (;;) {
+            if (nl > DL - 32) {
+                flush_runs<0, 0, IPL, PHI, COMP, SAFE, false>(tile, LA, nl, eps2, I);
+                entries += nl;
+                nl = 0;
+                __syncwarp();
+                // over the quota: cut here, with no leaf pending and a stack
+                // that a record can hold
+                if (over_quota(a, entries + (QUAD ? qentries : 0), ng) && pbase >= pend && sp <= kHeavyStack) break;
+            }
+            if constexpr (QUAD) {
+                if (nq > DQ - 32) {
+                    flush_runs<0, 0, IPL, PHI, COMP, SAFE, true>(tile, LQ, nq, eps2, I);
+                    qentries += nq;
+                    nq = 0;
+                    __syncwarp();
+                    if (over_quota(a, entries + qentries, ng) && pbase >= pend && sp <= kHeavyStack) break;
+                }
+            }
+            if (pbase < pend) {
+                // ---- the next 32 pending particles.  Leaves are in increasing
+                // start order, so the owner of slot s is the last leaf starting
+                // at or before it: those before pbase plus the starts from
+                // there up to this lane
+                const int s = pbase + (int)lane;
+                const unsigned rel = (unsigned)(lexcl - pbase);  // lanes without a leaf: lexcl huge
+                const unsigned smap = __reduce_or_sync(NB_FULL, rel < 32u ? 1u << rel : 0u);
+                const int before = __popc(__ballot_sync(NB_FULL, lexcl < pbase));
+                const int k = before + __popc(smap & (0xffffffffu >> (31 - lane))) - 1;
+                const int of = __shfl_sync(NB_FULL, ldelta, k & 31);
+                if (s < pend) list_put(LA, nl + (int)lane, __ldg(&a.pos4[of + s]));
+                nl += min(32, pend - pbase);
+                pbase += 32;
+                __syncwarp();
+                continue;
+            }
+            if (sp <= 0) break;
             // ---- pop the top four child ranges (<= 8 nodes each): lane L takes
             // node L % 8 of range L / 8.  Opened internal nodes have close to 8
             // children, so the lanes stay nearly full without a scan of the
@@ -487,7 +576,7 @@ __global__ void __maxnreg__(walk_regs<IPL>()) walk_kernel(WalkArgs a, int geomet
             if (rr < take) e = stk[sp - 1 - rr];
             const int node = (int)(e >> 3) + jj;
             const bool slot = rr < take && jj <= (int)(e & 7u);
-            const bool in_range = node >= 0 && node < nnodes;
+            const bool in_range = (unsigned)node < (unsigned)nnodes;
             if (slot && !in_range) bad = true;
             const bool has = slot && in_range;
             sp -= take;
@@ -513,18 +602,17 @@ __global__ void __maxnreg__(walk_regs<IPL>()) walk_kernel(WalkArgs a, int geomet
             // children sit on the next level, so their ids exceed the parent's:
             // a descent that does not increase the id would be a corrupt tree
             const bool bad_link = has && !accept && !leaf &&
-                                  (link <= node || mcount < 1 || mcount > 8 || link + mcount > nnodes);
+                                  (link <= node || (unsigned)(mcount - 1) > 7u || link + mcount > nnodes);
             if (bad_link) bad = true;
             const bool open_node = has && !accept && !leaf && !bad_link;
 
             // ---- push the child ranges of opened internal nodes
             const unsigned om = __ballot_sync(NB_FULL, open_node);
-            const int npush = __popc(om);
             if (open_node) {
                 const int pos = sp + __popc(om & lt);
                 if (pos < S) stk[pos] = ((uint32_t)link << 3) | (uint32_t)(mcount - 1);
             }
-            sp += npush;
+            sp += __popc(om);
             if (sp > S) {
                 overflow = true;
                 sp = S;
@@ -533,37 +621,20 @@ __global__ void __maxnreg__(walk_regs<IPL>()) walk_kernel(WalkArgs a, int geomet
 
             // ---- accepted nodes join the list (with quadrupoles: the node list)
             const unsigned am = __ballot_sync(NB_FULL, accept);
-            const int na = __popc(am);
             if constexpr (QUAD) {
-                if (nq + na > DQ) {
-                    __syncwarp();
-                    flush_runs<0, 0, IPL, PHI, COMP, SAFE, true>(tile, LQ, nq, eps2, I);
-                    qentries += nq;
-                    nq = 0;
-                    __syncwarp();
-                }
                 if (accept)
                     quad_put(LQ, nq + __popc(am & lt), A, __ldg(&a.nodeQ[2 * node]),
                              __ldg(&a.nodeQ[2 * node + 1]));
-                nq += na;
+                nq += __popc(am);
             } else {
-                if (nl + na > D) {
-                    __syncwarp();
-                    flush_runs<0, 0, IPL, PHI, COMP, SAFE, false>(tile, LA, nl, eps2, I);
-                    entries += nl;
-                    nl = 0;
-                    __syncwarp();
-                }
                 if (accept) list_put(LA, nl + __popc(am & lt), A);
-                nl += na;
+                nl += __popc(am);
             }
 
-            // ---- particles of opened leaves join the list, 32 per chunk: the
-            // opened leaves are compacted to lanes 0..nlf-1 (through the warp's
-            // scratch words), their counts scanned, and each chunk's slots are
-            // mapped to their leaf with a bit map of the leaf starts, as in the
-            // pop above -- one load latency per 32 particles, not per leaf
-            const bool leaf_ok = open_leaf && link >= 0 && mcount >= 1 && link + mcount <= npart;
+            // ---- opened leaves become pending: compacted to lanes 0..nlf-1
+            // (through the warp's scratch words), their counts scanned
+            const bool leaf_ok = open_leaf && (unsigned)link < (unsigned)npart &&
+                                 (unsigned)(mcount - 1) < (unsigned)(npart - link);
             if (open_leaf && !leaf_ok) bad = true;
             const unsigned lm = __ballot_sync(NB_FULL, leaf_ok);
             if (lm) {
@@ -575,30 +646,10 @@ __global__ void __maxnreg__(walk_regs<IPL>()) walk_kernel(WalkArgs a, int geomet
                 const int lcs = __shfl_sync(NB_FULL, mcount, src);
                 const int lc = (int)lane < nlf ? lcs : 0;
                 const int lincl = warp_incl_scan(lc);
-                const int lexcl = lincl - lc;
-                const int total = __shfl_sync(NB_FULL, lincl, 31);
-                for (int base = 0; base < total; base += 32) {
-                    const int c = (total - base) < 32 ? (total - base) : 32;
-                    if (nl + c > D) {
-                        __syncwarp();
-                        flush_runs<0, 0, IPL, PHI, COMP, SAFE, false>(tile, LA, nl, eps2, I);
-                        entries += nl;
-                        nl = 0;
-                        __syncwarp();
-                    }
-                    // leaves are in increasing start order with counts >= 1, so
-                    // the owner of slot base+lane is the last leaf starting at
-                    // or before it: those before the chunk plus the starts
-                    // inside it up to this lane
-                    const bool starts = lc > 0 && lexcl >= base && lexcl < base + 32;
-                    const unsigned smap = __reduce_or_sync(NB_FULL, starts ? 1u << (lexcl - base) : 0u);
-                    const int before = __popc(__ballot_sync(NB_FULL, lc > 0 && lexcl < base));
-                    const int k = before + __popc(smap & (0xffffffffu >> (31 - lane))) - 1;
-                    const int of = __shfl_sync(NB_FULL, lf, k & 31);
-                    const int oex = __shfl_sync(NB_FULL, lexcl, k & 31);
-                    if ((int)lane < c) list_put(LA, nl + lane, __ldg(&a.pos4[of + base + (int)lane - oex]));
-                    nl += c;
-                }
+                pend = __shfl_sync(NB_FULL, lincl, 31);
+                pbase = 0;
+                lexcl = (int)lane < nlf ? lincl - lc : 0x7fffffff;
+                ldelta = lf - (lincl - lc);
             }
             __syncwarp();
         }
@@ -618,9 +669,14 @@ __global__ void __maxnreg__(walk_regs<IPL>()) walk_kernel(WalkArgs a, int geomet
         }
         __syncwarp();
 
-        finish_group<IPL, PHI, COMP, SAFE>(tile, first, cnt, eps2, a, I);
+        if (sp > 0) save_heavy(a, ds, g, sp, entries + qentries, stk);
+        const float G = sp > 0 ? 1.0f : a.G;
+        const float self = SAFE || sp > 0 ? 0.0f : rsqrt_fast(eps2);
+        group_sums<IPL, PHI, COMP>(tile, cnt, I, [&](int idx, const float (&r)[4], float mi) {
+            store_force<PHI>(a, first + idx, r, mi, G, self);
+        });
         entries += qentries;
-        if (lane == 0 && a.grp_cost) a.grp_cost[g] = (int32_t)entries;
+        if (lane == 0 && a.grp_cost) a.grp_cost[g] = entries;
         warp_entries += (unsigned long long)entries;
         warp_inter += (unsigned long long)entries * (unsigned long long)cnt;
         warp_quad += (unsigned long long)qentries * (unsigned long long)cnt;
@@ -638,10 +694,18 @@ __global__ void __maxnreg__(walk_regs<IPL>()) walk_kernel(WalkArgs a, int geomet
 }
 
 template <int IPL, bool QUAD>
-cudaError_t launch_walk_ipl(cudaStream_t s, const WalkArgs &a, const WalkShape &sh, int nsm) {
+cudaError_t launch_walk_ipl(cudaStream_t s, const WalkArgs &args, const WalkShape &sh, int nsm) {
     const int threads = 32 * sh.warps_per_block;
-    const size_t smem =
-        (size_t)sh.warps_per_block * walk_smem_per_warp(a.list_depth, a.stack_depth, QUAD);
+    // a step's 32 entries of room beyond the list's depth where they fit (the
+    // list is then flushed when it holds at least list_depth entries, else
+    // up to 31 entries before: 0.5 % of the walk at depth 256)
+    WalkArgs a = args;
+    a.list_slack = 32;
+    size_t smem = (size_t)sh.warps_per_block * walk_smem_per_warp(a.list_depth, a.stack_depth, QUAD, 32);
+    if (smem > 227 * 1024) {
+        a.list_slack = 0;
+        smem = (size_t)sh.warps_per_block * walk_smem_per_warp(a.list_depth, a.stack_depth, QUAD);
+    }
     void (*k)(WalkArgs, int);
     if (sh.potential) {
         if (sh.compensated) k = sh.safe ? walk_kernel<IPL, true, true, true, QUAD> : walk_kernel<IPL, true, true, false, QUAD>;
