@@ -70,6 +70,7 @@ struct nbody_ctx {
     DevBuf sys_off, sys_box, sys_boxord, sys_eps2, sys_eps, sys_root;
     // walk / step
     DevBuf acc_s, aold_s;
+    const float *aold_cur = nullptr;  // |a_old| of the last walk where it is not in aold_s
     // cooperative walk: records of groups cut at the quota, partial sums of
     // groups walked in parts
     DevBuf heavy, cut, part, part_ctl;
@@ -306,7 +307,8 @@ cudaError_t ensure_capacity(nbody_ctx *c, int64_t n, int nsys, int levels) {
         NB_E(ensure(c->rs_temp, std::max(radix_temp_bytes(n), nosort_temp_bytes(n))));
         NB_E(ensure(c->tree_temp, tree_temp_bytes(n, kMaxLevels)));
         NB_E(ensure(c->grp_temp, (size_t)((n + 4095) / 4096 + 64) * 4));
-        NB_E(ensure(c->gflag, n));
+        NB_E(ensure(c->gflag, (n + 15) / 16 * 16));
+        NB_E(cudaMemsetAsync(c->gflag.p, 0, c->gflag.bytes, c->stream));  // every build leaves it zero
         NB_E(ensure(c->grp_first, n * 4)); NB_E(ensure(c->grp_count, n * 4));
         NB_E(ensure(c->grp_sphere, n * 16)); NB_E(ensure(c->grp_sys, n * 4));
         NB_E(ensure(c->grp_alpha, n * 4)); NB_E(ensure(c->grp_cost, n * 4));
@@ -326,10 +328,13 @@ cudaError_t ensure_capacity(nbody_ctx *c, int64_t n, int nsys, int levels) {
     }
     if (nsys > c->cap_sys) {
         NB_E(ensure(c->sys_off, (size_t)(nsys + 1) * 8)); NB_E(ensure(c->sys_box, (size_t)nsys * sizeof(SysBox)));
-        NB_E(ensure(c->sys_boxord, (size_t)nsys * 24)); NB_E(ensure(c->sys_eps2, (size_t)nsys * 4));
+        NB_E(ensure(c->sys_boxord, (size_t)nsys * 24 + 4)); NB_E(ensure(c->sys_eps2, (size_t)nsys * 4));
         NB_E(ensure(c->sys_eps, (size_t)nsys * 4));
         NB_E(ensure(c->sys_root, (size_t)nsys * 4));
         c->cap_sys = nsys;
+        // empty extents and a zero count of blocks: every build leaves them so
+        launch_bbox_init(c->stream, nsys, P<uint32_t>(c->sys_boxord));
+        NB_E(cudaMemsetAsync(P<uint32_t>(c->sys_boxord) + (size_t)nsys * 6, 0, 4, c->stream));
     }
 #undef NB_E
     return cudaSuccess;
@@ -363,9 +368,16 @@ nbody_status build_core(nbody_ctx *c, const Layout &L, const void *x, const void
                         bool near_order = false, const uint32_t *hint = nullptr) {
     cudaStream_t s = c->stream;
     launch_bbox(s, L, x, y, z, dbl, P<int64_t>(c->sys_off), P<uint32_t>(c->sys_boxord),
-                P<SysBox>(c->sys_box), c->nsm);
-    c->kernels += 3;
-    if (near_order && nosort_fits(L.n)) {
+                P<SysBox>(c->sys_box), P<uint32_t>(c->sys_boxord) + (size_t)c->cap_sys * 6, c->nsm);
+    c->kernels += bbox_kernels(L.nsys);
+    if (L.n <= kRankSortMax) {
+        launch_keys(s, L, x, y, z, dbl, P<int64_t>(c->sys_off), P<SysBox>(c->sys_box),
+                    P<uint64_t>(c->keys), P<uint32_t>(c->vals), nullptr, c->nsm);
+        NB_CUDA(c, rank_sort(s, P<uint64_t>(c->keys), L.n, P<uint64_t>(c->keys_alt), P<uint32_t>(c->vals_alt)));
+        c->kernels += 2;
+        std::swap(c->keys, c->keys_alt);
+        std::swap(c->vals, c->vals_alt);
+    } else if (near_order && nosort_fits(L.n)) {
         launch_keys(s, L, x, y, z, dbl, P<int64_t>(c->sys_off), P<SysBox>(c->sys_box),
                     P<uint64_t>(c->keys), P<uint32_t>(c->vals), nullptr, c->nsm);
         nosort(s, P<uint64_t>(c->keys), P<uint64_t>(c->keys_alt), P<uint32_t>(c->vals),
@@ -412,7 +424,9 @@ const uint32_t *first_sort_hint(const nbody_ctx *c, const Layout &L) {
                : nullptr;
 }
 
-nbody_status build_tree_groups(nbody_ctx *c, const Layout &L) {
+// aold (nullable): |a_old| in the new sorted order, for the groups' alpha; the
+// walk that follows then has nothing left to prepare.
+nbody_status build_tree_groups(nbody_ctx *c, const Layout &L, const float *aold = nullptr) {
     cudaStream_t s = c->stream;
     c->costs_valid = false;
     build_tree(s, L, P<uint64_t>(c->keys), P<float4>(c->pos4), P<SysBox>(c->sys_box),
@@ -426,18 +440,17 @@ nbody_status build_tree_groups(nbody_ctx *c, const Layout &L) {
                  P<int32_t>(c->node_start), P<int32_t>(c->node_parent), P<int32_t>(c->node_count),
                  P<int32_t>(c->node_nchild), P<int32_t>(c->node_link), c->ds,
                  P<uint8_t>(c->gflag), c->grp_temp.p, P<int32_t>(c->grp_first),
-                 P<int32_t>(c->grp_count), P<float4>(c->grp_sphere), P<int32_t>(c->grp_sys),
-                 c->nsm);
-    // tree: leaflevel, level scan, level offsets, node zeroing, nodes, two
-    // system-root kernels, moments; groups: 5
-    c->kernels += 8 + 5;
+                 P<int32_t>(c->grp_count), P<float4>(c->grp_sphere), P<int32_t>(c->grp_sys), aold,
+                 c->cfg.delta_acc, P<float>(c->grp_alpha), c->nsm);
+    // tree: leaflevel, level scan, node zeroing, nodes, moments
+    c->kernels += 5 + group_kernels(L.n);
     NB_CUDA(c, cudaGetLastError());
     return NBODY_OK;
 }
 
 // Refit of the current tree to the positions now in pos4 (sorted order):
 // moments with the child-recurrence b_J, then the group spheres.
-nbody_status refit_tree_groups(nbody_ctx *c, const Layout &L) {
+nbody_status refit_tree_groups(nbody_ctx *c, const Layout &L, const float *aold = nullptr) {
     cudaStream_t s = c->stream;
     c->costs_valid = false;
     tree_moments(s, L, P<uint64_t>(c->keys), P<float4>(c->pos4), P<SysBox>(c->sys_box),
@@ -449,7 +462,7 @@ nbody_status refit_tree_groups(nbody_ctx *c, const Layout &L) {
                  true);
     refit_groups(s, L, c->cfg.group_size, P<float4>(c->pos4), P<int64_t>(c->sys_off), c->ds,
                  P<int32_t>(c->grp_first), P<int32_t>(c->grp_count), P<float4>(c->grp_sphere),
-                 P<int32_t>(c->grp_sys), c->nsm);
+                 P<int32_t>(c->grp_sys), aold, c->cfg.delta_acc, P<float>(c->grp_alpha), c->nsm);
     c->kernels += 1 + 1;
     NB_CUDA(c, cudaGetLastError());
     return NBODY_OK;
@@ -670,11 +683,12 @@ WalkArgs walk_args(nbody_ctx *c, bool geometric) {
     return a;
 }
 
-// Reset the walk's queue head and counters (status is kept).
-nbody_status reset_walk_counters(nbody_ctx *c, bool accumulators) {
+// Reset the walk's queues (unless the group pass did) and counters (status is
+// kept).
+nbody_status reset_walk_counters(nbody_ctx *c, bool queues, bool accumulators) {
     char *base = reinterpret_cast<char *>(c->ds);
-    static_assert(offsetof(DevState, ncut) == offsetof(DevState, queue_head) + 4 * sizeof(int32_t), "adjacent");
-    NB_CUDA(c, cudaMemsetAsync(base + offsetof(DevState, queue_head), 0, 5 * sizeof(int32_t), c->stream));
+    if (queues)
+        NB_CUDA(c, cudaMemsetAsync(base + offsetof(DevState, queue), 0, sizeof(WalkQueue), c->stream));
     if (accumulators) {
         NB_CUDA(c, cudaMemsetAsync(base + offsetof(DevState, max_stack), 0, sizeof(int32_t), c->stream));
         NB_CUDA(c, cudaMemsetAsync(base + offsetof(DevState, list_entries), 0,
@@ -720,7 +734,7 @@ cudaError_t ensure_mlp_buffers(nbody_ctx *c) {
 
 void launch_features(nbody_ctx *c) {
     launch_mlp_features(c->stream, c->L, c->ds, P<int32_t>(c->grp_first), P<int32_t>(c->grp_count),
-                        P<float4>(c->grp_sphere), P<int32_t>(c->grp_sys), P<float>(c->aold_s),
+                        P<float4>(c->grp_sphere), P<int32_t>(c->grp_sys), c->aold_cur ? c->aold_cur : P<float>(c->aold_s),
                         P<uint64_t>(c->keys), P<float4>(c->nodeA), P<int32_t>(c->sys_root),
                         P<SysBox>(c->sys_box), P<int64_t>(c->sys_off), P<float>(c->feat), c->nsm);
     c->kernels += 1;
@@ -767,19 +781,22 @@ nbody_status compute_order(nbody_ctx *c, const float *pcost, const int32_t **ord
     return NBODY_OK;
 }
 
-// Walk over the current groups; aold_s (sorted) must hold |a_old|.
+// Walk over the current groups; aold_s (sorted) must hold |a_old|, unless the
+// group pass has formed alpha and reset the queues already (prepared).
 nbody_status run_walk(nbody_ctx *c, bool geometric, bool phi, bool safe, const int32_t *perm,
                       float *ax, float *ay, float *az, float *ph, float4 *acc_sorted,
                       bool reset_accumulators = true, const float *pcost = nullptr,
-                      const int32_t *active_order = nullptr, const int32_t *nactive = nullptr) {
+                      const int32_t *active_order = nullptr, const int32_t *nactive = nullptr,
+                      bool prepared = false) {
     const int32_t *order = active_order;
     if (!geometric && !active_order) {
         nbody_status so = compute_order(c, pcost, &order);
         if (so != NBODY_OK) return so;
     }
-    nbody_status st = reset_walk_counters(c, reset_accumulators);
+    // (the alpha pass resets the queues too)
+    nbody_status st = reset_walk_counters(c, geometric, reset_accumulators);
     if (st != NBODY_OK) return st;
-    if (!geometric) {
+    if (!geometric && !prepared) {
         launch_group_alpha(c->stream, c->L.n, c->ds, P<int32_t>(c->grp_first),
                            P<int32_t>(c->grp_count), P<float>(c->aold_s), c->cfg.delta_acc,
                            P<float>(c->grp_alpha), c->nsm);
@@ -814,7 +831,7 @@ nbody_status run_walk(nbody_ctx *c, bool geometric, bool phi, bool safe, const i
         NB_CUDA(c, cudaEventRecordWithFlags(c->gwev[c->gwev_used + 1], c->stream, cudaEventRecordExternal));
         c->gwev_used += 2;
     }
-    c->kernels += c->L.n <= kCoopParticles ? 1 : 2;
+    c->kernels += (c->L.n <= kCoopParticles ? 1 : 2) + (c->L.n > kCutQuota ? 1 : 0);
     if (!geometric) c->costs_valid = true;
     return NBODY_OK;
 }
@@ -1007,6 +1024,7 @@ nbody_status nbody_walk(nbody_ctx *ctx, const float *a_old, float *ax, float *ay
     NB_CUDA(ctx, cudaMemsetAsync(dsb + offsetof(DevState, status), 0, sizeof(int32_t), s));
     NB_CUDA(ctx, cudaEventRecord(ctx->ev[2], s));
     nbody_status st;
+    ctx->aold_cur = nullptr;
     if (a_old) {
         const void *dao;
         NB_CUDA(ctx, stage_in(ctx, 8, a_old, fb, &dao));
@@ -1174,10 +1192,10 @@ static nbody_status block_steps(nbody_ctx *ctx, const Layout &L, StepState *S, i
                 ctx->kernels += 2;
             }
             cur = 1 - cur;
-            st = build_tree_groups(ctx, L);
+            st = build_tree_groups(ctx, L, S[cur].aold);
             rebuilds++;
         } else {
-            st = refit_tree_groups(ctx, L);
+            st = refit_tree_groups(ctx, L, S[cur].aold);
         }
         if (st != NBODY_OK) return st;
         NB_CUDA(ctx, pool_event(ctx, &e1));
@@ -1189,7 +1207,7 @@ static nbody_status block_steps(nbody_ctx *ctx, const Layout &L, StepState *S, i
                                    S[cur].lvl, T, K, P<int32_t>(ctx->grp_order), dact, ctx->nsm);
         ctx->kernels += 1;
         st = run_walk(ctx, false, false, safe, nullptr, nullptr, nullptr, nullptr, nullptr, acc,
-                      false, nullptr, P<int32_t>(ctx->grp_order), dact);
+                      false, nullptr, P<int32_t>(ctx->grp_order), dact, true);
         if (st != NBODY_OK) return st;
         NB_CUDA(ctx, pool_event(ctx, &e2));
         NB_CUDA(ctx, cudaEventRecord(e2, q));
@@ -1234,6 +1252,7 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
     if (st != NBODY_OK) return st;
     const bool safe = any_zero_eps(ctx, nsys, eps_sys);
     ctx->L = L;  // the walk's bounds checks read the particle count from here
+    ctx->aold_cur = nullptr;
     StepState S[2];
     for (int b = 0; b < 2; b++) {
         S[b].x = P<double>(ctx->st_buf[b][0]);
@@ -1287,10 +1306,10 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
     // positions, which the kick-drift writes to pos4 in place).
     int rebuilds = 0;
     // A step defers its closing half kick into the next step's kick-drift
-    // pass (pending_kick): between eager steps, and between the two steps of
-    // a graph; the graph's last step kicks on its own, so that every replay
-    // starts from the same state.
-    bool pending_kick = false, defer_in_capture = false;
+    // pass (pending_kick), or into the store at the call's end: the first step
+    // and every graph replay end with one pending, so every replay starts from
+    // the same state.
+    bool pending_kick = false;
     // near_order: the state is in the Morton order of this call's previous
     // build (every step but the call's first, whose state is in caller order)
     auto one_step = [&](bool timing, bool rebuild, bool near_order) -> nbody_status {
@@ -1324,19 +1343,27 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
             loaded_recs = false;
             ctx->kernels += 1;
             cur = 1 - cur;
-            r = build_tree_groups(ctx, L);
+            r = build_tree_groups(ctx, L, S[cur].aold);
             rebuilds++;
         } else {
-            r = refit_tree_groups(ctx, L);
+            r = refit_tree_groups(ctx, L, S[cur].aold);
         }
         if (r != NBODY_OK) return r;
         if (timing) {
             NB_CUDA(ctx, pool_event(ctx, &e1));
             NB_CUDA(ctx, cudaEventRecord(e1, q));
         }
-        NB_CUDA(ctx, cudaMemcpyAsync(ctx->aold_s.p, S[cur].aold, fb, cudaMemcpyDeviceToDevice, q));
+        // the cost model's features read |a_old| of this walk: in place, as the
+        // state keeps it until the next step -- except when a kick follows
+        // here (dt = 0) and sets the next one
+        if (dt == 0.0f) {
+            NB_CUDA(ctx, cudaMemcpyAsync(ctx->aold_s.p, S[cur].aold, fb, cudaMemcpyDeviceToDevice, q));
+            ctx->aold_cur = nullptr;
+        } else {
+            ctx->aold_cur = S[cur].aold;
+        }
         r = run_walk(ctx, false, false, safe, nullptr, nullptr, nullptr, nullptr, nullptr, acc, false,
-                     S[cur].pcost);
+                     S[cur].pcost, nullptr, nullptr, true);
         if (r != NBODY_OK) return r;
         if (S[cur].pcost) {
             launch_spread_cost(q, &ctx->ds->ngroups, P<int32_t>(ctx->grp_first),
@@ -1349,7 +1376,7 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
             NB_CUDA(ctx, cudaEventRecord(e2, q));
             marks.push_back(ctx->evused - 3);
         }
-        if ((ctx->capturing && !defer_in_capture) || dt == 0.0f) {
+        if (dt == 0.0f) {
             launch_kick(q, n, S[cur], acc, 0.5f * dt);
             ctx->kernels += 1;
         } else {
@@ -1369,11 +1396,6 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
         // of the build before them.
         st = one_step(true, true, false);
         if (st != NBODY_OK) return st;
-        if (pending_kick) {
-            launch_kick(s, n, S[cur], acc, 0.5f * dt);
-            ctx->kernels += 1;
-            pending_kick = false;
-        }
         sorted_state = true;
         // Two steps per graph: the sort's ping-pong buffers and the state
         // copies swap roles every step, so after two steps every pointer is
@@ -1413,9 +1435,7 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
             cudaError_t ce = cudaStreamBeginCapture(ctx->gstream, cudaStreamCaptureModeRelaxed);
             nbody_status r1 = NBODY_OK, r2 = NBODY_OK;
             if (ce == cudaSuccess) {
-                defer_in_capture = true;
                 r1 = one_step(false, true, true);
-                defer_in_capture = false;
                 if (r1 == NBODY_OK) r2 = one_step(false, true, true);
                 cudaError_t ee = cudaStreamEndCapture(ctx->gstream, &graph);
                 if (ce == cudaSuccess) ce = ee;

@@ -37,17 +37,22 @@ constexpr int kStatusStackOverflow = 1;
 constexpr int kStatusBadTree = 2;  // an index failed a bounds check (skipped)
 constexpr int kStatusTimeout = 4;  // a bounded device wait ran out (results invalid)
 
+// Queues of one walk, reset together before it.
+struct WalkQueue {
+    int32_t head;
+    int32_t coop_head[2];
+    int32_t nheavy;  // groups cut at the quota by the current walk
+    int32_t ncut;    // parts cut by the cooperative walk's first stage
+};
+
 // Device-resident counters and small per-build values.
 struct DevState {
     int32_t nnodes;
     int32_t ngroups;
-    int32_t queue_head;  // walk queues: reset together before every walk
-    int32_t coop_head[2];
-    int32_t nheavy;      // groups cut at the quota by the current walk
-    int32_t ncut;        // parts cut by the cooperative walk's first stage
+    WalkQueue queue;
     int32_t status;
     int32_t max_stack;
-    int32_t pad0;
+    int32_t scan_done;  // blocks of the level scan that have finished
     unsigned long long list_entries;
     unsigned long long interactions;
     unsigned long long quad_entries;  // list entries that were quadrupole nodes
@@ -142,7 +147,12 @@ __device__ __forceinline__ int sys_of(const int64_t *off, int nsys, int64_t i) {
 // ---------------------------------------------------------------- launchers
 // sort.cu
 void launch_bbox(cudaStream_t s, const Layout &L, const void *x, const void *y, const void *z,
-                 bool dbl, const int64_t *d_off, uint32_t *d_boxord, SysBox *d_box, int nsm);
+                 bool dbl, const int64_t *d_off, uint32_t *d_boxord, SysBox *d_box, uint32_t *d_done,
+                 int nsm);
+// Empties the extents of nsys systems (a new buffer; launch_bbox leaves them
+// empty, and *d_done zero).
+void launch_bbox_init(cudaStream_t s, int nsys, uint32_t *d_boxord);
+int bbox_kernels(int nsys);
 // Morton keys (vals = 0..n-1).  With sort_temp (cleared by radix_prepare),
 // the kernel also accumulates the radix sort's digit histograms, and the
 // sort is then called with hist_done = true.
@@ -183,6 +193,10 @@ void nosort(cudaStream_t s, uint64_t *keys, uint64_t *kout, uint32_t *vscr, uint
 void nosort_hint_gather(cudaStream_t s, int64_t n, const uint64_t *keys, const uint32_t *hint,
                         uint64_t *kout, uint32_t *vout);
 int nosort_kernels();
+// The stable sort of up to kRankSortMax keys below 2^63 in any order, in one
+// launch: kout the sorted keys, vout the input index of each.
+constexpr int kRankSortMax = 8192;
+cudaError_t rank_sort(cudaStream_t s, const uint64_t *keys, int64_t n, uint64_t *kout, uint32_t *vout);
 // True for memory the current device dev can read in place (its own device
 // memory, or managed memory); diag_noalloc.cu.
 bool on_device(const void *p, int dev);
@@ -214,13 +228,19 @@ void tree_moments(cudaStream_t s, const Layout &L, const uint64_t *keys, const f
                   float4 *nodeQ, int nsm, bool refit);
 void refit_groups(cudaStream_t s, const Layout &L, int group_size, const float4 *pos4,
                   const int64_t *d_off, DevState *ds, const int32_t *grp_first,
-                  int32_t *grp_count, float4 *grp_sphere, int32_t *grp_sys, int nsm);
+                  int32_t *grp_count, float4 *grp_sphere, int32_t *grp_sys, const float *aold,
+                  float dacc, float *grp_alpha, int nsm);
+// gflag: uint8 [n rounded up to 16], zero before and after.  aold (nullable,
+// sorted): the groups' alpha too, and the walk's queues are reset.
 void build_groups(cudaStream_t s, const Layout &L, int group_size, const float4 *pos4,
                   const int64_t *d_off, const int32_t *node_start, const int32_t *node_parent,
                   const int32_t *node_count, const int32_t *node_nchild, const int32_t *node_link,
                   DevState *ds, uint8_t *gflag, void *temp, int32_t *grp_first,
-                  int32_t *grp_count, float4 *grp_sphere, int32_t *grp_sys, int nsm);
-void launch_group_alpha(cudaStream_t s, int64_t n, const DevState *ds, const int32_t *grp_first,
+                  int32_t *grp_count, float4 *grp_sphere, int32_t *grp_sys, const float *aold,
+                  float dacc, float *grp_alpha, int nsm);
+int group_kernels(int64_t n);
+// Also resets the walk's queues.
+void launch_group_alpha(cudaStream_t s, int64_t n, DevState *ds, const int32_t *grp_first,
                         const int32_t *grp_count, const float *aold_sorted, float delta_acc,
                         float *grp_alpha, int nsm);
 

@@ -24,11 +24,18 @@ namespace nb {
 // Per-system bounding box: each warp keeps running min/max while its chunks
 // stay in one system, the block merges its warps, and one set of atomics per
 // (block, system) publishes the result.
+__device__ void bbox_finalize(int s, int levels, uint32_t *boxord, SysBox *box);
+
+// done != nullptr: the block that finishes last also turns the extents into
+// cubes and empties them for the next build, so the cube is one launch (of
+// about 3 us each at N = 4096) instead of three; with many systems a kernel of
+// its own does that with more than one block.
 template <typename T>
 __global__ void __launch_bounds__(256) bbox_kernel(int64_t n, const T *__restrict__ x,
                                                    const T *__restrict__ y, const T *__restrict__ z,
                                                    const int64_t *__restrict__ off, int nsys,
-                                                   uint32_t *boxord) {
+                                                   uint32_t *boxord, int levels, SysBox *box,
+                                                   uint32_t *done) {
     __shared__ float sh_lo[8][3], sh_hi[8][3];
     __shared__ int sh_s[8];
     const unsigned lane = lane_id(), w = threadIdx.x >> 5;
@@ -125,8 +132,19 @@ __global__ void __launch_bounds__(256) bbox_kernel(int64_t n, const T *__restric
             }
         }
     }
+    if (!done) return;
+    __shared__ int last;
+    __threadfence();  // this thread's extents before the block counts itself in
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int s = threadIdx.x; s < nsys; s += blockDim.x) bbox_finalize(s, levels, boxord, box);
+    if (threadIdx.x == 0) *done = 0;
 }
 
+// No extent yet (a new buffer; afterwards every build leaves it so).
 __global__ void bbox_init_kernel(int nsys, uint32_t *boxord) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nsys * 6; i += gridDim.x * blockDim.x)
         boxord[i] = (i % 6) < 3 ? 0xffffffffu : 0u;
@@ -135,37 +153,55 @@ __global__ void bbox_init_kernel(int nsys, uint32_t *boxord) {
 // Cube of each system, in FP32 with the stated operation order:
 // corner = per-axis minimum; L = (max extent) * (1 + 2^-20); L = 1 if 0;
 // scale = 2^levels / L.
-__global__ void bbox_finalize_kernel(int nsys, int levels, const uint32_t *boxord, SysBox *box) {
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nsys; s += gridDim.x * blockDim.x) {
-        SysBox b;
-        if (boxord[s * 6] == 0xffffffffu) {  // empty system
-            b.x0 = b.y0 = b.z0 = 0.0f;
-            b.L = 1.0f;
-        } else {
-            float lo[3], hi[3];
-            for (int a = 0; a < 3; a++) {
-                lo[a] = ord2f(boxord[s * 6 + a]);
-                hi[a] = ord2f(boxord[s * 6 + 3 + a]);
-            }
-            float ext = __fsub_rn(hi[0], lo[0]);
-            float ey = __fsub_rn(hi[1], lo[1]), ez = __fsub_rn(hi[2], lo[2]);
-            if (ey > ext) ext = ey;
-            if (ez > ext) ext = ez;
-            float L = __fmul_rn(ext, 1.0f + 0x1p-20f);
-            b.x0 = lo[0];
-            b.y0 = lo[1];
-            b.z0 = lo[2];
-            b.L = (L > 0.0f) ? L : 1.0f;
-        }
-        b.scale = __fdiv_rn((float)(1u << levels), b.L);
-        b.pad[0] = b.pad[1] = b.pad[2] = 0.0f;
-        box[s] = b;
+__device__ void bbox_finalize(int s, int levels, uint32_t *boxord, SysBox *box) {
+    uint32_t o[6];
+    for (int a = 0; a < 6; a++) {
+        o[a] = __ldcg(&boxord[s * 6 + a]);
+        boxord[s * 6 + a] = a < 3 ? 0xffffffffu : 0u;
     }
+    SysBox b;
+    if (o[0] == 0xffffffffu) {  // empty system
+        b.x0 = b.y0 = b.z0 = 0.0f;
+        b.L = 1.0f;
+    } else {
+        float lo[3], hi[3];
+        for (int a = 0; a < 3; a++) {
+            lo[a] = ord2f(o[a]);
+            hi[a] = ord2f(o[3 + a]);
+        }
+        float ext = __fsub_rn(hi[0], lo[0]);
+        float ey = __fsub_rn(hi[1], lo[1]), ez = __fsub_rn(hi[2], lo[2]);
+        if (ey > ext) ext = ey;
+        if (ez > ext) ext = ez;
+        float L = __fmul_rn(ext, 1.0f + 0x1p-20f);
+        b.x0 = lo[0];
+        b.y0 = lo[1];
+        b.z0 = lo[2];
+        b.L = (L > 0.0f) ? L : 1.0f;
+    }
+    b.scale = __fdiv_rn((float)(1u << levels), b.L);
+    b.pad[0] = b.pad[1] = b.pad[2] = 0.0f;
+    box[s] = b;
 }
 
+__global__ void bbox_finalize_kernel(int nsys, int levels, uint32_t *boxord, SysBox *box) {
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nsys; s += gridDim.x * blockDim.x)
+        bbox_finalize(s, levels, boxord, box);
+}
+
+void launch_bbox_init(cudaStream_t s, int nsys, uint32_t *boxord) {
+    bbox_init_kernel<<<(nsys * 6 + 255) / 256, 256, 0, s>>>(nsys, boxord);
+}
+
+// One block of 256 threads turns up to 2048 systems' extents into cubes in a
+// few steps; more take the kernel of their own.
+constexpr int kBoxLast = 2048;
+int bbox_kernels(int nsys) { return nsys <= kBoxLast ? 1 : 2; }
+
 void launch_bbox(cudaStream_t s, const Layout &L, const void *x, const void *y, const void *z,
-                 bool dbl, const int64_t *d_off, uint32_t *d_boxord, SysBox *d_box, int nsm) {
-    bbox_init_kernel<<<(L.nsys * 6 + 255) / 256, 256, 0, s>>>(L.nsys, d_boxord);
+                 bool dbl, const int64_t *d_off, uint32_t *d_boxord, SysBox *d_box, uint32_t *d_done,
+                 int nsm) {
+    if (L.nsys > kBoxLast) d_done = nullptr;
     int64_t warps = (L.n + 255) / 256;
     int blocks = (int)((warps + 7) / 8);
     int maxb = nsm * NB_SCAN_CTAS_PER_SM;
@@ -173,11 +209,14 @@ void launch_bbox(cudaStream_t s, const Layout &L, const void *x, const void *y, 
     if (blocks < 1) blocks = 1;
     if (dbl)
         bbox_kernel<double><<<blocks, 256, 0, s>>>(L.n, (const double *)x, (const double *)y,
-                                                   (const double *)z, d_off, L.nsys, d_boxord);
+                                                   (const double *)z, d_off, L.nsys, d_boxord,
+                                                   L.levels, d_box, d_done);
     else
         bbox_kernel<float><<<blocks, 256, 0, s>>>(L.n, (const float *)x, (const float *)y,
-                                                  (const float *)z, d_off, L.nsys, d_boxord);
-    bbox_finalize_kernel<<<(L.nsys + 127) / 128, 128, 0, s>>>(L.nsys, L.levels, d_boxord, d_box);
+                                                  (const float *)z, d_off, L.nsys, d_boxord,
+                                                  L.levels, d_box, d_done);
+    if (!d_done)
+        bbox_finalize_kernel<<<(L.nsys + 127) / 128, 128, 0, s>>>(L.nsys, L.levels, d_boxord, d_box);
 }
 
 // ---------------------------------------------------------------- Morton keys

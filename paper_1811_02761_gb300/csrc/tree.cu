@@ -120,12 +120,13 @@ __global__ void __launch_bounds__(TB) leaflevel_kernel(Layout L, int cap,
 }
 
 // One block per level: exclusive scan of that level's block counts; the
-// level's node count goes to lvl_off[l + 1] (turned into offsets below).
+// level's node count goes to lvl_off[l + 1], and the block that finishes last
+// turns the counts into offsets.
 // Each thread scans LS_IPT consecutive counts, so a level of 32768 blocks
 // takes four block-wide scans.
 constexpr int LS_T = 1024, LS_IPT = 8;
 __global__ void __launch_bounds__(LS_T) level_scan_kernel(uint32_t *blockcnt, int nblk,
-                                                          DevState *ds) {
+                                                          DevState *ds, int64_t cap_nodes) {
     __shared__ uint32_t sh[32];
     const int l = blockIdx.x;
     const int w = threadIdx.x >> 5;
@@ -153,25 +154,30 @@ __global__ void __launch_bounds__(LS_T) level_scan_kernel(uint32_t *blockcnt, in
         carry += sh[31];
         __syncthreads();
     }
-    if (threadIdx.x == 0) ds->lvl_off[l + 1] = (int32_t)carry;
-}
-
-__global__ void level_offsets_kernel(int NL, DevState *ds, int64_t cap_nodes) {
     if (threadIdx.x != 0) return;
+    ds->lvl_off[l + 1] = (int32_t)carry;
+    __threadfence();
+    if (atomicAdd(&ds->scan_done, 1) != (int)gridDim.x - 1) return;
+    __threadfence();
     int32_t off = 0;
     ds->lvl_off[0] = 0;
-    for (int l = 0; l < NL; l++) {
-        off += ds->lvl_off[l + 1];
-        ds->lvl_off[l + 1] = off;
+    for (int k = 0; k < (int)gridDim.x; k++) {
+        off += __ldcg(&ds->lvl_off[k + 1]);
+        ds->lvl_off[k + 1] = off;
     }
     ds->nnodes = off;
+    ds->scan_done = 0;
     if (off > cap_nodes) atomicOr(&ds->status, kStatusStackOverflow);
 }
 
 // Zeroes the child counts and the moments pass's arrival counters of the
-// nodes about to be made (the node count is on the device).
+// nodes about to be made (the node count is on the device); no system has a
+// root yet.
 __global__ void node_zero_kernel(const DevState *__restrict__ ds, int64_t cap_nodes,
-                                 int32_t *node_nchild, int32_t *node_arrive) {
+                                 int32_t *node_nchild, int32_t *node_arrive, int nsys,
+                                 int32_t *sys_root) {
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nsys; s += gridDim.x * blockDim.x)
+        sys_root[s] = -1;
     const int64_t nn = min((int64_t)ds->nnodes, cap_nodes);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nn;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -196,7 +202,9 @@ __global__ void __launch_bounds__(TB) nodes_kernel(Layout L, const int8_t *__res
                                                    int64_t cap_nodes, int32_t *node_start,
                                                    int8_t *node_level, int32_t *node_parent,
                                                    int32_t *node_link, int32_t *node_count,
-                                                   int32_t *node_nchild) {
+                                                   int32_t *node_nchild,
+                                                   const int64_t *__restrict__ off,
+                                                   int32_t *sys_root) {
     __shared__ uint32_t wc[kMaxNL][TB / 32];
     __shared__ int32_t sbase[kMaxNL];
     const int64_t n = L.n;
@@ -253,6 +261,7 @@ __global__ void __launch_bounds__(TB) nodes_kernel(Layout L, const int8_t *__res
             const int par = prev_id >= 0 ? prev_id : (di >= 0 ? pex - 1 : -1);
             node_parent[id] = par;
             if (par >= 0) atomicAdd(&node_nchild[par], 1);
+            if (l == 0) sys_root[sys_of(off, L.nsys, i)] = id;
             if (l == Li) {  // leaf: particles until the next boundary above level l
                 int64_t j = i + 1;
                 while (j < n && delta[j] >= l) j++;
@@ -262,18 +271,6 @@ __global__ void __launch_bounds__(TB) nodes_kernel(Layout L, const int8_t *__res
         }
         prev_id = id;
     }
-}
-
-__global__ void sys_root_kernel(const DevState *ds, const int32_t *node_start, const int64_t *off,
-                                int nsys, int32_t *sys_root) {
-    int nroot = ds->lvl_off[1];
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nroot; r += gridDim.x * blockDim.x)
-        sys_root[sys_of(off, nsys, node_start[r])] = r;
-}
-
-__global__ void sys_root_init_kernel(int nsys, int32_t *sys_root) {
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nsys; s += gridDim.x * blockDim.x)
-        sys_root[s] = -1;
 }
 
 // ---------------------------------------------------------------- moments
@@ -646,13 +643,13 @@ void build_tree(cudaStream_t s, const Layout &L, const uint64_t *keys, const flo
         leaflevel_kernel<16><<<(nblk + VB - 1) / VB, TB, 0, s>>>(L, leaf_cap, keys, delta, leaflev, blockcnt, nblk);
     else
         leaflevel_kernel<32><<<(nblk + VB - 1) / VB, TB, 0, s>>>(L, leaf_cap, keys, delta, leaflev, blockcnt, nblk);
-    level_scan_kernel<<<L.levels + 1, LS_T, 0, s>>>(blockcnt, nblk, ds);
-    level_offsets_kernel<<<1, 32, 0, s>>>(L.levels + 1, ds, cap_nodes);
-    node_zero_kernel<<<nsm * 8, 256, 0, s>>>(ds, cap_nodes, node_nchild, node_arrive);
+    level_scan_kernel<<<L.levels + 1, LS_T, 0, s>>>(blockcnt, nblk, ds, cap_nodes);
+    int zb = (int)((L.n + 255) / 256);  // the nodes are fewer than the particles, mostly
+    if (zb > nsm * 8) zb = nsm * 8;
+    node_zero_kernel<<<zb, 256, 0, s>>>(ds, cap_nodes, node_nchild, node_arrive, L.nsys, sys_root);
     nodes_kernel<<<nblk, TB, 0, s>>>(L, delta, leaflev, blockcnt, nblk, ds, cap_nodes, node_start,
-                                     node_level, node_parent, node_link, node_count, node_nchild);
-    sys_root_init_kernel<<<(L.nsys + 255) / 256, 256, 0, s>>>(L.nsys, sys_root);
-    sys_root_kernel<<<(L.nsys + 255) / 256, 256, 0, s>>>(ds, node_start, d_off, L.nsys, sys_root);
+                                     node_level, node_parent, node_link, node_count, node_nchild,
+                                     d_off, sys_root);
     tree_moments(s, L, keys, pos4, d_box, leaf_cap, G, ds, node_start, node_level, node_parent,
                  node_link, node_count, node_nchild, node_arrive, nodeA, nodeB, mass2, nodeQ, nsm,
                  false);
@@ -764,7 +761,8 @@ __global__ void __launch_bounds__(FL_T) flag_count_kernel(const uint8_t *__restr
     }
 }
 
-__global__ void __launch_bounds__(FL_T) flag_write_kernel(const uint8_t *__restrict__ f, int64_t n,
+// Writes the groups' first particles and clears the flags for the next build.
+__global__ void __launch_bounds__(FL_T) flag_write_kernel(uint8_t *__restrict__ f, int64_t n,
                                                           const uint32_t *__restrict__ bsum,
                                                           int32_t *__restrict__ out) {
     __shared__ uint32_t sh[32];
@@ -776,19 +774,55 @@ __global__ void __launch_bounds__(FL_T) flag_write_kernel(const uint8_t *__restr
     }
     uint32_t ex = block_excl_scan_1024(t, sh) + bsum[blockIdx.x];
     for (int k = 0; k < FL_IPT; k++) {
-        if (v[k]) out[ex] = (int32_t)(base + k);
+        if (v[k]) {
+            out[ex] = (int32_t)(base + k);
+            f[base + k] = 0;
+        }
         ex += v[k];
     }
 }
 
-// Warp per group: count, bounding-box centre and enclosing radius, system.
+// Count, scan and write in one block, for up to kFlagOne particles: one launch
+// instead of three, 16 flags per thread and step.
+constexpr int kFlagOne = 1 << 16;
+__global__ void __launch_bounds__(FL_T) flag_one_kernel(uint8_t *__restrict__ f, int n,
+                                                        int32_t *__restrict__ out, int32_t *total) {
+    __shared__ uint32_t sh[32];
+    uint32_t carry = 0;
+    for (int b0 = 0; b0 < n; b0 += FL_T * 16) {
+        const int base = b0 + (int)threadIdx.x * 16;  // f has room to the next multiple of 16
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (base < n) v = *reinterpret_cast<uint4 *>(f + base);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        const uint32_t t = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);  // flags are 0 or 1
+        uint32_t ex = carry + block_excl_scan_1024(t, sh);
+        if (t) {
+            *reinterpret_cast<uint4 *>(f + base) = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                for (uint32_t m = w[k]; m; m &= m - 1) out[ex++] = base + 4 * k + ((__ffs(m) - 1) >> 3);
+        }
+        if (threadIdx.x == FL_T - 1) sh[0] = ex;
+        __syncthreads();
+        carry = sh[0];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *total = (int32_t)carry;
+}
+
+// Warp per group: count, bounding-box centre and enclosing radius, system;
+// with aold also alpha (as group_alpha_kernel), and with queue the walk's
+// queues are reset: a step's walk then needs no launch of its own for either.
 __global__ void __launch_bounds__(256) group_info_kernel(Layout L, int G,
                                                          const float4 *__restrict__ pos4,
                                                          const int64_t *__restrict__ off,
                                                          const DevState *__restrict__ ds,
                                                          const int32_t *__restrict__ grp_first,
                                                          int32_t *grp_count, float4 *grp_sphere,
-                                                         int32_t *grp_sys) {
+                                                         int32_t *grp_sys,
+                                                         const float *__restrict__ aold, float dacc,
+                                                         float *grp_alpha, WalkQueue *queue) {
+    if (queue && blockIdx.x == 0 && threadIdx.x == 0) *queue = WalkQueue{};
     // a half-warp per group, two groups per warp at a time: both groups'
     // member loads are in flight together (min, max and the largest distance
     // do not depend on the order of the reduction)
@@ -805,9 +839,11 @@ __global__ void __launch_bounds__(256) group_info_kernel(Layout L, int G,
             cnt = end - first;
         }
         float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+        float amin = INFINITY;
 #pragma unroll 4
         for (int k = (int)sl; k < cnt; k += 16) {
             float4 p = pos4[first + k];
+            if (aold) amin = fminf(amin, aold[first + k]);
             lo[0] = fminf(lo[0], p.x); hi[0] = fmaxf(hi[0], p.x);
             lo[1] = fminf(lo[1], p.y); hi[1] = fmaxf(hi[1], p.y);
             lo[2] = fminf(lo[2], p.z); hi[2] = fmaxf(hi[2], p.z);
@@ -827,7 +863,10 @@ __global__ void __launch_bounds__(256) group_info_kernel(Layout L, int G,
             r2 = fmaxf(r2, dx * dx + dy * dy + dz * dz);
         }
         for (int o = 8; o; o >>= 1) r2 = fmaxf(r2, __shfl_xor_sync(NB_FULL, r2, o));
+        if (aold)
+            for (int o = 8; o; o >>= 1) amin = fminf(amin, __shfl_xor_sync(NB_FULL, amin, o));
         if (sl == 0 && g < ng) {
+            if (aold) grp_alpha[g] = dacc * amin;
             // rounded up so the sphere encloses every member despite FP32 error
             float r = __fsqrt_ru(r2) * (1.0f + 0x1p-20f);
             grp_count[g] = cnt;
@@ -841,37 +880,46 @@ void build_groups(cudaStream_t s, const Layout &L, int group_size, const float4 
                   const int64_t *d_off, const int32_t *node_start, const int32_t *node_parent,
                   const int32_t *node_count, const int32_t *node_nchild, const int32_t *node_link,
                   DevState *ds, uint8_t *gflag, void *temp, int32_t *grp_first,
-                  int32_t *grp_count, float4 *grp_sphere, int32_t *grp_sys, int nsm) {
-
-    cudaMemsetAsync(gflag, 0, (size_t)L.n, s);
+                  int32_t *grp_count, float4 *grp_sphere, int32_t *grp_sys, const float *aold,
+                  float dacc, float *grp_alpha, int nsm) {
     int mb = (int)((L.n + 255) / 256);
     if (mb > nsm * 16) mb = nsm * 16;
     group_mark_kernel<<<mb, 256, 0, s>>>(ds, group_size, node_start, node_parent, node_link, node_count,
                                          node_nchild, gflag);
-    int nb = (int)((L.n + FL_CH - 1) / FL_CH);
-    uint32_t *bsum = (uint32_t *)temp;
-    flag_count_kernel<<<nb, FL_T, 0, s>>>(gflag, L.n, bsum);
-    launch_scan_sums(s, bsum, nb, &ds->ngroups);
-    flag_write_kernel<<<nb, FL_T, 0, s>>>(gflag, L.n, bsum, grp_first);
-    int gb = nsm * NB_GROUP_CTAS_PER_SM;
-    group_info_kernel<<<gb, 256, 0, s>>>(L, group_size, pos4, d_off, ds, grp_first, grp_count,
-                                         grp_sphere, grp_sys);
+    if (L.n <= kFlagOne) {
+        flag_one_kernel<<<1, FL_T, 0, s>>>(gflag, (int)L.n, grp_first, &ds->ngroups);
+    } else {
+        int nb = (int)((L.n + FL_CH - 1) / FL_CH);
+        uint32_t *bsum = (uint32_t *)temp;
+        flag_count_kernel<<<nb, FL_T, 0, s>>>(gflag, L.n, bsum);
+        launch_scan_sums(s, bsum, nb, &ds->ngroups);
+        flag_write_kernel<<<nb, FL_T, 0, s>>>(gflag, L.n, bsum, grp_first);
+    }
+    refit_groups(s, L, group_size, pos4, d_off, ds, grp_first, grp_count, grp_sphere, grp_sys, aold, dacc,
+                 grp_alpha, nsm);
 }
+
+int group_kernels(int64_t n) { return n <= kFlagOne ? 3 : 5; }
 
 // Spheres (and counts, systems) of the existing groups from pos4: after a
 // refit the membership stays and only the geometry is recomputed.
 void refit_groups(cudaStream_t s, const Layout &L, int group_size, const float4 *pos4,
                   const int64_t *d_off, DevState *ds, const int32_t *grp_first,
-                  int32_t *grp_count, float4 *grp_sphere, int32_t *grp_sys, int nsm) {
-    group_info_kernel<<<nsm * NB_GROUP_CTAS_PER_SM, 256, 0, s>>>(L, group_size, pos4, d_off, ds, grp_first, grp_count,
-                                              grp_sphere, grp_sys);
+                  int32_t *grp_count, float4 *grp_sphere, int32_t *grp_sys, const float *aold,
+                  float dacc, float *grp_alpha, int nsm) {
+    int gb = (int)((L.n + 255) / 256);  // 16 groups per CTA and step, of at least a few particles
+    if (gb > nsm * NB_GROUP_CTAS_PER_SM) gb = nsm * NB_GROUP_CTAS_PER_SM;
+    group_info_kernel<<<gb, 256, 0, s>>>(L, group_size, pos4, d_off, ds, grp_first, grp_count,
+                                         grp_sphere, grp_sys, aold, dacc, grp_alpha,
+                                         aold ? &ds->queue : nullptr);
 }
 
 // alpha_g = delta_acc * min over members of |a_old| (Eq. 2 per group).
-__global__ void group_alpha_kernel(const DevState *__restrict__ ds,
+__global__ void group_alpha_kernel(DevState *ds,
                                    const int32_t *__restrict__ grp_first,
                                    const int32_t *__restrict__ grp_count,
                                    const float *__restrict__ aold, float dacc, float *grp_alpha) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ds->queue = WalkQueue{};
     // a half-warp per group, two groups per warp at a time (as group_info)
     const int ng = ds->ngroups;
     const unsigned lane = lane_id(), sl = lane & 15u;
@@ -892,12 +940,12 @@ __global__ void group_alpha_kernel(const DevState *__restrict__ ds,
     }
 }
 
-void launch_group_alpha(cudaStream_t s, int64_t n, const DevState *ds, const int32_t *grp_first,
+void launch_group_alpha(cudaStream_t s, int64_t n, DevState *ds, const int32_t *grp_first,
                         const int32_t *grp_count, const float *aold_sorted, float delta_acc,
                         float *grp_alpha, int nsm) {
-    (void)n;
-    group_alpha_kernel<<<nsm * NB_GROUP_CTAS_PER_SM, 256, 0, s>>>(ds, grp_first, grp_count, aold_sorted, delta_acc,
-                                                grp_alpha);
+    int gb = (int)((n + 255) / 256);
+    if (gb > nsm * NB_GROUP_CTAS_PER_SM) gb = nsm * NB_GROUP_CTAS_PER_SM;
+    group_alpha_kernel<<<gb, 256, 0, s>>>(ds, grp_first, grp_count, aold_sorted, delta_acc, grp_alpha);
 }
 
 }  // namespace nb

@@ -82,7 +82,7 @@ __global__ void __maxnreg__(walk_regs<IPL>())
     unsigned long long cta_entries = 0, cta_inter = 0, cta_quad = 0;
 
     const bool all = !second && ng <= a.coop_groups;
-    const int T = second ? ds->ncut : (all ? ng : min(ds->nheavy, a.heavy_cap));
+    const int T = second ? ds->queue.ncut : (all ? ng : min(ds->queue.nheavy, a.heavy_cap));
     const int P = T > 0 ? max(1, min(kCoopParts, a.coop_target[second] / T)) : 1;
     const bool may_cut = !second && T <= kCutTasks / P;
 
@@ -110,7 +110,7 @@ __global__ void __maxnreg__(walk_regs<IPL>())
             for (int k = tid; k < sp; k += 32 * W) stk[k] = rec[kHeavyHead + k];
         }
         if (tid == 0)  // read after the walk
-            s_task = (int)gridDim.x + atomicAdd(&ds->coop_head[second], 1);
+            s_task = (int)gridDim.x + atomicAdd(&ds->queue.coop_head[second], 1);
         long long entries = 0, qentries = 0;
         bool shared = P > 1;  // the top of the tree, expanded by every part of the group
         int nf = 0;
@@ -314,7 +314,7 @@ __global__ void __maxnreg__(walk_regs<IPL>())
         const int owner = second ? (int)rec[2] : rec_i * P;
         if (sp > 0) {  // cut: the open ranges become a record of the second stage
             if (tid == 0) {
-                const int k = s_cut = atomicAdd(&ds->ncut, 1);  // k < T P <= kCutTasks
+                const int k = s_cut = atomicAdd(&ds->queue.ncut, 1);  // k < T P <= kCutTasks
                 a.cut_of[task] = k;
                 atomicAdd(&a.cut_count[owner], 1);
             }

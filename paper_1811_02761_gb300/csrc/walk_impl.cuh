@@ -444,7 +444,7 @@ __device__ __forceinline__ void load_sums(const WalkArgs &a, int i, float (&r)[4
 static __device__ __noinline__ void save_heavy(const WalkArgs &a, DevState *ds, int g, int sp, int entries, const uint32_t *stk) {
     const int lane = (int)lane_id();
     int h = 0;
-    if (lane == 0) h = atomicAdd(&ds->nheavy, 1);
+    if (lane == 0) h = atomicAdd(&ds->queue.nheavy, 1);
     h = __shfl_sync(NB_FULL, h, 0);
     uint32_t *rec = a.heavy + (size_t)h * kHeavyWords;  // h < ng <= heavy_cap
     if (lane == 0) {
@@ -505,7 +505,7 @@ __global__ void __maxnreg__(walk_regs<IPL>()) walk_kernel(WalkArgs a, int geomet
 
     for (;;) {
         int qi = 0;
-        if (lane == 0) qi = atomicAdd(&ds->queue_head, 1);
+        if (lane == 0) qi = atomicAdd(&ds->queue.head, 1);
         qi = __shfl_sync(NB_FULL, qi, 0);
         if (qi >= ng) break;
         const int g = a.order ? a.order[qi] : qi;
