@@ -159,11 +159,14 @@ __global__ void __launch_bounds__(LS_T) level_scan_kernel(uint32_t *blockcnt, in
     __threadfence();
     if (atomicAdd(&ds->scan_done, 1) != (int)gridDim.x - 1) return;
     __threadfence();
-    int32_t off = 0;
+    int32_t cnt[kMaxNL], off = 0;  // all loads before the first store
+#pragma unroll
+    for (int k = 0; k < kMaxNL; k++) cnt[k] = k < (int)gridDim.x ? __ldcg(&ds->lvl_off[k + 1]) : 0;
     ds->lvl_off[0] = 0;
-    for (int k = 0; k < (int)gridDim.x; k++) {
-        off += __ldcg(&ds->lvl_off[k + 1]);
-        ds->lvl_off[k + 1] = off;
+#pragma unroll
+    for (int k = 0; k < kMaxNL; k++) {
+        off += cnt[k];
+        if (k < (int)gridDim.x) ds->lvl_off[k + 1] = off;
     }
     ds->nnodes = off;
     ds->scan_done = 0;
@@ -369,83 +372,103 @@ __device__ __forceinline__ void write_quad(int id, const float q[6], float4 *nod
 // from zero too; a node that fails its bounds check is still counted in at
 // its parent, which keeps every counter consistent.
 
-// One internal node from its children's records (contiguous, at most 8), by
-// one thread.  Sums run over the children in octant order, relative to the
-// cell centre; the size is
+// One internal node per team of eight lanes from its children's records
+// (contiguous, at most 8), a lane per child; every lane of the warp calls this
+// (go false: a team without a node).  Sums are reduced over the team pairwise,
+// relative to the cell centre; the size is
 //   b = min(max_c (|com_c - com| + b_c), distance from com to the farthest
 //           corner of the cell widened by one finest cell),
 // rounded up.  After a refit (positions moved since the build, members may
 // have left the cell) only the child recurrence bounds b.  Children finished
 // by other SMs in this launch are read past L1 (ld.global.cg): a sibling's
 // cache line may already sit in this SM's L1 from before it was written.
-__device__ __forceinline__ bool internal_node(const Layout &L, int p, int c0, int nc, int level,
-                                              uint64_t key, int refit, int nn,
-                                              const SysBox *__restrict__ box, float G,
-                                              int32_t *node_count, float4 *nodeA, float4 *nodeB,
-                                              float2 *mass2, float4 *nodeQ) {
-    if (c0 <= p || nc < 1 || nc > 8 || c0 + nc > nn) return false;
-    const CellF cell = node_cell(L, key, level, box);
-    // every field of every child in one round trip; the positions and sizes
-    // stay in registers for the size bound
-    float CX[8], CY[8], CZ[8], CB[8];
+// Bound by latency, as a climb is a chain of these: one thread per node, with
+// its 32 loads, eight square roots and eight-term double-float chain one after
+// the other, made the whole pass 35 us at n = 4096 and 47 us at 100003 (ncu);
+// with eight lanes it is 30 and 39 us.
+// Records of a small tree's nodes in shared memory (moments_one_kernel).
+struct NodeRec {
+    float4 A;
+    float2 M;
+    int count;
+    float b;
+};
+__device__ __forceinline__ bool internal_nodes(const Layout &L, bool go, int p, int c0, int nc,
+                                               int level, uint64_t key, int refit, int nn,
+                                               const SysBox *__restrict__ box, float G,
+                                               int32_t *node_count, float4 *nodeA, float4 *nodeB,
+                                               float2 *mass2, float4 *nodeQ, NodeRec *rec_s = nullptr) {
+    const bool ok = go && !(c0 <= p || nc < 1 || nc > 8 || c0 + nc > nn);
+    const int sub = (int)(lane_id() & 7u);
+    const bool has = ok && sub < nc;
+    float4 A = make_float4(0.f, 0.f, 0.f, 0.f), q0 = A, q1 = A;
     float2 M = make_float2(0.0f, 0.0f);
-    float px = 0.0f, py = 0.0f, pz = 0.0f;
     int count = 0;
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const int j = k < nc ? c0 + k : c0;
-        const float4 A = __ldcg(nodeA + j);
-        const float2 mk = __ldcg(mass2 + j);
-        const int ck = __ldcg(node_count + j);
-        CB[k] = __ldcg(&nodeB[j].x);
-        CX[k] = A.x; CY[k] = A.y; CZ[k] = A.z;
-        if (k < nc) {
-            M = df_add(M, mk);
-            count += ck;
-            px = fmaf(A.w, A.x - cell.c[0], px);
-            py = fmaf(A.w, A.y - cell.c[1], py);
-            pz = fmaf(A.w, A.z - cell.c[2], pz);
+    float b = 0.0f;
+    if (has) {  // every field in one round trip
+        const int j = c0 + sub;
+        if (rec_s) {
+            const NodeRec r = rec_s[j];
+            A = r.A;
+            M = r.M;
+            count = r.count;
+            b = r.b;
+        } else {
+            A = __ldcg(nodeA + j);
+            M = __ldcg(mass2 + j);
+            count = __ldcg(node_count + j);
+            b = __ldcg(&nodeB[j].x);
         }
+        if (nodeQ) {
+            q0 = __ldcg(nodeQ + 2 * j);
+            q1 = __ldcg(nodeQ + 2 * j + 1);
+        }
+    }
+    CellF cell{};
+    if (ok) cell = node_cell(L, key, level, box);
+    const float w = A.w;
+    float px = w * (A.x - cell.c[0]), py = w * (A.y - cell.c[1]), pz = w * (A.z - cell.c[2]);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        const float2 Mo = make_float2(__shfl_xor_sync(NB_FULL, M.x, o), __shfl_xor_sync(NB_FULL, M.y, o));
+        M = df_add(M, Mo);
+        px += __shfl_xor_sync(NB_FULL, px, o);
+        py += __shfl_xor_sync(NB_FULL, py, o);
+        pz += __shfl_xor_sync(NB_FULL, pz, o);
+        count += __shfl_xor_sync(NB_FULL, count, o);
     }
     float cp[3] = {cell.c[0], cell.c[1], cell.c[2]};
     if (M.x > 0.0f) {
         const float inv = 1.0f / M.x;
         cp[0] = fmaf(px, inv, cp[0]); cp[1] = fmaf(py, inv, cp[1]); cp[2] = fmaf(pz, inv, cp[2]);
     }
-    float rec = 0.0f;
-    float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const float dx = A.x - cp[0], dy = A.y - cp[1], dz = A.z - cp[2];
+    const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+    float rec = has ? __fadd_ru(__fsqrt_ru(r2), b) : 0.0f;
 #pragma unroll
-    for (int k = 0; k < 8; k++) {
-        if (k < nc) {
-            const float dx = CX[k] - cp[0], dy = CY[k] - cp[1], dz = CZ[k] - cp[2];
-            const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-            rec = fmaxf(rec, __fadd_ru(__fsqrt_ru(r2), CB[k]));
-        }
-    }
+    for (int o = 1; o < 8; o <<= 1) rec = fmaxf(rec, __shfl_xor_sync(NB_FULL, rec, o));
+    float q[6] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y};
     if (nodeQ) {
+        if (has) quad_add(q, w, dx, dy, dz, r2);
 #pragma unroll
-        for (int k = 0; k < 8; k++) {
-            if (k >= nc) break;
-            const int j = c0 + k;
-            const float4 A = __ldcg(nodeA + j);
-            const float dx = A.x - cp[0], dy = A.y - cp[1], dz = A.z - cp[2];
-            const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-            const float4 q0 = __ldcg(nodeQ + 2 * j), q1 = __ldcg(nodeQ + 2 * j + 1);
-            q[0] += q0.x; q[1] += q0.y; q[2] += q0.z; q[3] += q0.w; q[4] += q1.x; q[5] += q1.y;
-            quad_add(q, A.w, dx, dy, dz, r2);
+        for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+            for (int k = 0; k < 6; k++) q[k] += __shfl_xor_sync(NB_FULL, q[k], o);
+    }
+    if (ok && sub == 0) {
+        float c2 = 0.0f;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const float e = fabsf(cp[a] - cell.c[a]) + cell.h;
+            c2 = fmaf(e, e, c2);
         }
+        const float bp = (refit ? rec : fminf(rec, __fsqrt_ru(c2))) * kUp;
+        node_count[p] = count;
+        write_node(p, cp[0], cp[1], cp[2], M, bp, G, c0, nc << 1, nodeA, nodeB, mass2);
+        if (rec_s) rec_s[p] = NodeRec{make_float4(cp[0], cp[1], cp[2], M.x), M, count, bp};
+        if (nodeQ) write_quad(p, q, nodeQ);
     }
-    float c2 = 0.0f;
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const float e = fabsf(cp[a] - cell.c[a]) + cell.h;
-        c2 = fmaf(e, e, c2);
-    }
-    const float bp = (refit ? rec : fminf(rec, __fsqrt_ru(c2))) * kUp;
-    node_count[p] = count;
-    write_node(p, cp[0], cp[1], cp[2], M, bp, G, c0, nc << 1, nodeA, nodeB, mass2);
-    if (nodeQ) write_quad(p, q, nodeQ);
-    return true;
+    return ok || !go;
 }
 
 // Count a finished node in at its parent `par` (one atomic add with release
@@ -601,24 +624,149 @@ __global__ void __launch_bounds__(256, NB_MOMENTS_MIN_CTAS) moments_kernel(
             level = lev0;
             key = key0;
         }
-        while (par >= 0) {       // a root has none
-            if (par >= node) {   // parents precede their children
-                bad = true;
-                break;
+        for (;;) {
+            bool ready = false;
+            int c0 = 0, nc = 0, up = -1;
+            if (par >= 0) {  // a root has none
+                if (par >= node) {  // parents precede their children
+                    bad = true;
+                } else {
+                    // the parent's fields load beside the count-in atomic; the
+                    // lane that brings the last child has the parent computed
+                    c0 = node_link[par];
+                    nc = node_nchild[par];
+                    up = node_parent[par];
+                    ready = count_in(par, node_arrive) == nc;
+                }
             }
-            // the parent's fields load beside the count-in atomic; the thread
-            // that brings the last child computes the parent
-            const int c0 = node_link[par], nc = node_nchild[par];
-            const int up = node_parent[par];
-            if (count_in(par, node_arrive) != nc) break;
-            level--;
-            if (!internal_node(L, par, c0, nc, level, key, refit, nn, box, G, node_count, nodeA,
-                               nodeB, mass2, nodeQ))
-                bad = true;  // still counted in above, so the counters stay consistent
-            node_arrive[par] = 0;
-            node = par;
-            par = up;
+            unsigned rm = __ballot_sync(NB_FULL, ready);
+            if (!rm) break;
+            while (rm) {  // four parents at a time, eight lanes each
+                int src = -1;
+#pragma unroll
+                for (int t = 0; t < 4; t++) {
+                    const int bit = rm ? __ffs(rm) - 1 : -1;
+                    rm &= rm - 1;
+                    if (t == (lane >> 3)) src = bit;
+                }
+                const int from = src >= 0 ? src : 0;
+                const int p = __shfl_sync(NB_FULL, par, from);
+                const int pc0 = __shfl_sync(NB_FULL, c0, from), pnc = __shfl_sync(NB_FULL, nc, from);
+                const int pl = __shfl_sync(NB_FULL, level, from) - 1;
+                const uint64_t pkey = __shfl_sync(NB_FULL, key, from);
+                if (!internal_nodes(L, src >= 0, p, pc0, pnc, pl, pkey, refit, nn, box, G, node_count,
+                                    nodeA, nodeB, mass2, nodeQ))
+                    bad = true;  // still counted in above, so the counters stay consistent
+            }
+            // the teams' records are device-visible before any lane counts one in
+            __threadfence();
+            __syncwarp();
+            if (ready) {
+                node_arrive[par] = 0;
+                node = par;
+                par = up;
+                level--;
+            } else {
+                par = -1;
+            }
         }
+    }
+    if (bad) atomicOr(&ds_status(ds), kStatusBadTree);
+}
+
+// The moments of a small tree by one block: the leaves (a thread each, as the
+// one-lane teams above: same operations, same order), then the internal nodes
+// level by level from the deepest, with the records in shared memory (a tree
+// of up to kOneNodes nodes) and block barriers where the pass above has L2
+// round trips, a fence and an atomic count per level.  At n = 4096 (1023 nodes,
+// 13 levels) that pass takes 30 us, almost all of it the climb's chain, and
+// this one 23 us (warm caches), most of it the leaves' own chains and the code's
+// first fetch.
+constexpr int kMomentsOne = 8192;  // particles; leaves of at most 16 members
+constexpr int kOneNodes = 4096;
+__global__ void __launch_bounds__(1024) moments_one_kernel(
+    Layout L, int refit, const uint64_t *__restrict__ keys, const float4 *__restrict__ pos4,
+    const SysBox *__restrict__ box, float G, DevState *ds, const int32_t *__restrict__ node_start,
+    const int8_t *__restrict__ node_level, const int32_t *__restrict__ node_link,
+    int32_t *node_count, const int32_t *__restrict__ node_nchild, float4 *nodeA, float4 *nodeB,
+    float2 *mass2, float4 *nodeQ) {
+    extern __shared__ __align__(16) unsigned char one_smem[];
+    __shared__ int s_off[kMaxNL + 1];
+    const int nn = ds->nnodes;
+    NodeRec *rec_s = nn <= kOneNodes ? reinterpret_cast<NodeRec *>(one_smem) : nullptr;
+    if (threadIdx.x <= L.levels + 1) s_off[threadIdx.x] = min(ds->lvl_off[threadIdx.x], nn);
+    bool bad = false;
+    for (int id = threadIdx.x; id < nn; id += blockDim.x) {
+        if (node_nchild[id] != 0) continue;
+        const int first = node_link[id], cnt = node_count[id];
+        if (first < 0 || cnt < 1 || (int64_t)first + cnt > L.n) {
+            bad = true;
+            continue;
+        }
+        const float4 r0 = pos4[first];
+        float2 M = make_float2(0.0f, 0.0f);
+        float sx = 0.0f, sy = 0.0f, sz = 0.0f;
+#pragma unroll 8
+        for (int k = 0; k < cnt; k++) {
+            const float4 p = pos4[first + k];
+            M = df_add(M, make_float2(p.w, 0.0f));
+            sx = fmaf(p.w, p.x - r0.x, sx);
+            sy = fmaf(p.w, p.y - r0.y, sy);
+            sz = fmaf(p.w, p.z - r0.z, sz);
+        }
+        float c[3] = {r0.x, r0.y, r0.z};
+        if (M.x > 0.0f) {
+            const float inv = 1.0f / M.x;
+            c[0] = fmaf(sx, inv, c[0]); c[1] = fmaf(sy, inv, c[1]); c[2] = fmaf(sz, inv, c[2]);
+        } else {
+            const CellF cell = node_cell(L, keys[node_start[id]], node_level[id], box);
+#pragma unroll
+            for (int a = 0; a < 3; a++) c[a] = cell.c[a];
+        }
+        float b2 = 0.0f;
+        float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+        for (int k = 0; k < cnt; k++) {
+            const float4 p = pos4[first + k];
+            const float dx = p.x - c[0], dy = p.y - c[1], dz = p.z - c[2];
+            const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+            b2 = fmaxf(b2, r2);
+            if (nodeQ) quad_add(q, p.w, dx, dy, dz, r2);
+        }
+        const float bl = __fsqrt_ru(b2) * kUp;
+        write_node(id, c[0], c[1], c[2], M, bl, G, first, (cnt << 1) | 1, nodeA, nodeB, mass2);
+        if (rec_s) rec_s[id] = NodeRec{make_float4(c[0], c[1], c[2], M.x), M, cnt, bl};
+        if (nodeQ) write_quad(id, q, nodeQ);
+    }
+    __syncthreads();
+    // a team of eight lanes per node; the fields the build wrote are loaded a
+    // level ahead, for the first nodes of each level
+    auto fields = [&](int id, int end, int &nc, int &c0, uint64_t &key) {
+        nc = id < end ? node_nchild[id] : 0;
+        c0 = id < end ? node_link[id] : 0;
+        key = id < end ? keys[node_start[id]] : 0ull;
+    };
+    const int team = (int)(threadIdx.x >> 3), teams = (int)(blockDim.x >> 3);
+    int fnc = 0, fc0 = 0;
+    uint64_t fkey = 0;
+    for (int l = L.levels; l >= 0; l--) {
+        const int n0 = s_off[l], n1 = s_off[l + 1];
+        const int nnc = fnc, nc0 = fc0;
+        const uint64_t nkey = fkey;
+        if (l > 0) fields(s_off[l - 1] + team, n0, fnc, fc0, fkey);  // the next level's first
+        if (n0 >= n1) continue;  // the same for every thread
+        for (int i0 = n0; i0 < n1; i0 += teams) {
+            const int id = i0 + team;
+            int nc = nnc, c0 = nc0;
+            uint64_t key = nkey;
+            if (i0 > n0 || l == L.levels) fields(id, n1, nc, c0, key);
+            // warps without a node stay out of the issue slots of the others
+            if (__any_sync(NB_FULL, nc > 0) &&
+                !internal_nodes(L, nc > 0, id, c0, nc, l, key, refit, nn, box, G, node_count, nodeA,
+                                nodeB, mass2, nodeQ, rec_s))
+                bad = true;
+        }
+        __syncthreads();
     }
     if (bad) atomicOr(&ds_status(ds), kStatusBadTree);
 }
@@ -674,6 +822,14 @@ void tree_moments(cudaStream_t s, const Layout &L, const uint64_t *keys, const f
                   const int32_t *node_link, int32_t *node_count, const int32_t *node_nchild,
                   int32_t *node_arrive, float4 *nodeA, float4 *nodeB, float2 *mass2,
                   float4 *nodeQ, int nsm, bool refit) {
+    if (L.n <= kMomentsOne && leaf_cap <= 16) {
+        const int smem = kOneNodes * (int)sizeof(NodeRec);
+        cudaFuncSetAttribute(moments_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        moments_one_kernel<<<1, 1024, smem, s>>>(L, refit ? 1 : 0, keys, pos4, d_box, G, ds, node_start,
+                                              node_level, node_link, node_count, node_nchild, nodeA,
+                                              nodeB, mass2, nodeQ);
+        return;
+    }
     int64_t mb = (L.n / 4 + 255) / 256;
     if (mb > (int64_t)nsm * NB_LEAF_CTAS_PER_SM) mb = (int64_t)nsm * NB_LEAF_CTAS_PER_SM;
     if (mb < 1) mb = 1;
