@@ -35,7 +35,7 @@ def sources():
 
 
 def _deps():
-    return (sources() + glob.glob(os.path.join(CSRC, "*.cuh")) +
+    return (sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) +
             [os.path.join(INCLUDE, "nbody.h"), os.path.abspath(__file__)])
 
 

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "scratch.h"
 
 using namespace nb;
 
@@ -925,6 +926,7 @@ nbody_status nbody_destroy(nbody_ctx *ctx) {
     if (ctx->gstream) cudaStreamDestroy(ctx->gstream);
     for (auto ev : ctx->evpool) cudaEventDestroy(ev);
     delete ctx;
+    nb::Scratch::give_back();
     return NBODY_OK;
 }
 
@@ -1832,7 +1834,7 @@ nbody_status nbody_mlp_train(nbody_ctx *ctx, int32_t epochs, float lr, int32_t b
     if (ng < 1) return fail(ctx, NBODY_EINVAL, "no groups");
     cudaStream_t s = ctx->stream;
     const int64_t nbatches = (ng + batch - 1) / batch;
-    const int maxb = (int)((ng / nbatches + 1 + 127) / 128) + 1;
+    const int maxb = (int)((ng / nbatches + 1 + kMlpGradBlock - 1) / kMlpGradBlock) + 1;
     cudaError_t e = ensure_mlp_buffers(ctx);
     if (e == cudaSuccess) e = ensure(ctx->mlp_gpart, (size_t)maxb * kMlpParams * 4);
     if (e == cudaSuccess) e = ensure(ctx->mlp_lpart, (size_t)maxb * 4);
@@ -1854,7 +1856,7 @@ nbody_status nbody_mlp_train(nbody_ctx *ctx, int32_t epochs, float lr, int32_t b
             const int count = (int)((ng - 1 - k) / nbatches + 1);
             ctx->mlp_t += 1;
             e = launch_mlp_train_step(s, P<float>(ctx->feat), P<float>(ctx->target), k, nbatches,
-                                      count, wb, P<float>(ctx->mlp_norm), P<float>(ctx->mlp_gpart),
+                                      count, wb, nullptr, P<float>(ctx->mlp_norm), P<float>(ctx->mlp_gpart),
                                       P<float>(ctx->mlp_lpart), nullptr,
                                       P<float>(ctx->mlp_loss) + k, P<float>(ctx->mlp_w),
                                       P<float>(ctx->mlp_m1), P<float>(ctx->mlp_m2), wb, lr,
@@ -1905,51 +1907,53 @@ nbody_status nbody_mlp_eval(int64_t n, const float *features, const float *targe
     if (n < 1 || n > (1 << 20) || !features || !targets || !params)
         return fail(nullptr, NBODY_EINVAL, "bad argument (1 <= n <= 2^20, non-NULL inputs)");
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const int nb = (int)((n + 127) / 128);
-    // one device block: features, targets, params, norm, pred, grad, partials, loss, bf16 params
+    const int nb = (int)((n + kMlpGradBlock - 1) / kMlpGradBlock);
     const size_t fsz = (size_t)n * 8 * 4, tsz = (size_t)n * 4, psz = kMlpParams * 4;
-    const size_t total = fsz + tsz + psz + 64 + tsz + psz + (size_t)nb * psz + (size_t)nb * 4 + 16 +
-                         kMlpParams * 2 + 1024;
-    char *buf = nullptr;
-    cudaError_t e = cudaMalloc(&buf, total);
-    if (e != cudaSuccess) return fail(nullptr, NBODY_ENOMEM, "allocation");
+    // Device arrays are read and written in place.  Host inputs are staged
+    // behind the partial sums; host outputs are written by the kernels into
+    // page-locked memory and copied from there (three copies into pageable
+    // memory took 100 us at n = 60013, allocating and freeing the device block
+    // another 100).
     auto align = [](size_t v) { return (v + 255) & ~(size_t)255; };
-    size_t o = 0;
-    float *dfeat = (float *)(buf + o); o = align(o + fsz);
-    float *dtarget = (float *)(buf + o); o = align(o + tsz);
-    float *dparams = (float *)(buf + o); o = align(o + psz);
-    float *dnorm = (float *)(buf + o); o = align(o + 64);
-    float *dpred = (float *)(buf + o); o = align(o + tsz);
-    float *dgrad = (float *)(buf + o); o = align(o + psz);
-    float *dgpart = (float *)(buf + o); o = align(o + (size_t)nb * psz);
-    float *dlpart = (float *)(buf + o); o = align(o + (size_t)nb * 4);
-    float *dloss = (float *)(buf + o); o = align(o + 16);
-    __nv_bfloat16 *dwb = (__nv_bfloat16 *)(buf + o);
-    auto h2d = [&](void *dst, const void *src, size_t b) {
-        return cudaMemcpyAsync(dst, src, b, is_device_ptr(src) ? cudaMemcpyDeviceToDevice
-                                                               : cudaMemcpyHostToDevice, s);
-    };
-    e = h2d(dfeat, features, fsz);
-    if (e == cudaSuccess) e = h2d(dtarget, targets, tsz);
-    if (e == cudaSuccess) e = h2d(dparams, params, psz);
-    if (e == cudaSuccess && norm) e = h2d(dnorm, norm, 64);
-    if (e == cudaSuccess) {
-        launch_mlp_round(s, dparams, dwb);
-        launch_mlp_forward(s, nullptr, n, dfeat, dwb, norm ? dnorm : nullptr, nullptr, dpred, 152);
-        e = launch_mlp_train_step(s, dfeat, dtarget, 0, 1, (int)n, dwb, norm ? dnorm : nullptr,
-                                  dgpart, dlpart, dgrad, dloss, nullptr, nullptr, nullptr, nullptr,
-                                  0.0f, 1, false);
+    size_t dev = align((size_t)nb * psz) + align((size_t)nb * 4), host = 0;
+    const void *in[4] = {features, targets, params, norm};
+    const size_t isz[4] = {fsz, tsz, psz, 64};
+    size_t ioff[4];
+    for (int k = 0; k < 4; k++) {
+        ioff[k] = in[k] && !is_device_ptr(in[k]) ? dev : SIZE_MAX;
+        if (ioff[k] != SIZE_MAX) dev += align(isz[k]);
     }
-    auto d2h = [&](void *dst, const void *src, size_t b) {
-        return cudaMemcpyAsync(dst, src, b, is_device_ptr(dst) ? cudaMemcpyDeviceToDevice
-                                                               : cudaMemcpyDeviceToHost, s);
-    };
-    if (e == cudaSuccess && pred) e = d2h(pred, dpred, tsz);
-    if (e == cudaSuccess && grad) e = d2h(grad, dgrad, psz);
-    if (e == cudaSuccess && loss) e = d2h(loss, dloss, 4);
+    void *out[3] = {pred, grad, loss};
+    const size_t osz[3] = {tsz, psz, 4};
+    size_t ooff[3];
+    for (int k = 0; k < 3; k++) {
+        ooff[k] = out[k] && !is_device_ptr(out[k]) ? host : SIZE_MAX;
+        if (ooff[k] != SIZE_MAX) host += align(osz[k]);
+    }
+    nb::Scratch scratch(s);
+    cudaError_t e = scratch.take(dev, host);
+    if (e != cudaSuccess) return fail(nullptr, NBODY_ENOMEM, "allocation");
+    float *gpart = reinterpret_cast<float *>(scratch.dev);
+    float *lpart = reinterpret_cast<float *>(scratch.dev + align((size_t)nb * psz));
+    const float *din[4];
+    for (int k = 0; k < 4 && e == cudaSuccess; k++) {
+        din[k] = static_cast<const float *>(in[k]);
+        if (ioff[k] == SIZE_MAX) continue;
+        din[k] = reinterpret_cast<const float *>(scratch.dev + ioff[k]);
+        e = cudaMemcpyAsync(scratch.dev + ioff[k], in[k], isz[k], cudaMemcpyHostToDevice, s);
+    }
+    float *dout[3];
+    for (int k = 0; k < 3; k++)
+        dout[k] = ooff[k] == SIZE_MAX ? static_cast<float *>(out[k])
+                                      : reinterpret_cast<float *>(scratch.host + ooff[k]);
+    if (e == cudaSuccess)
+        e = launch_mlp_train_step(s, din[0], din[1], 0, 1, (int)n, nullptr, din[2], din[3], gpart, lpart,
+                                  dout[1], dout[2], nullptr, nullptr, nullptr, nullptr, 0.0f, 1, false,
+                                  dout[0]);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(buf);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "nbody_mlp_eval");
+    for (int k = 0; k < 3; k++)
+        if (ooff[k] != SIZE_MAX) std::memcpy(out[k], scratch.host + ooff[k], osz[k]);
     return NBODY_OK;
 }
 

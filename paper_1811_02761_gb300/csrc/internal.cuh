@@ -356,12 +356,16 @@ void launch_mlp_features(cudaStream_t s, const Layout &L, const DevState *ds,
 void launch_mlp_forward(cudaStream_t s, const int32_t *pn, int64_t n, const float *feat,
                         const __nv_bfloat16 *wb, const float *norm, const float *tnorm,
                         float *pred, int nsm);
-size_t mlp_grad_smem();
+// gpart: kMlpParams floats and lpart: one per block of kMlpGradBlock samples.
+// The weights are wb, or w32 (not NULL) rounded to BF16; pred (nullable)
+// receives the network's output of every sample.
+constexpr int kMlpGradBlock = 64;
 cudaError_t launch_mlp_train_step(cudaStream_t s, const float *feat, const float *target,
                                   int64_t base, int64_t stride, int count,
-                                  const __nv_bfloat16 *wb, const float *norm, float *gpart,
-                                  float *lpart, float *grad, float *loss, float *w, float *m1,
-                                  float *m2, __nv_bfloat16 *wb_out, float lr, int t, bool update);
+                                  const __nv_bfloat16 *wb, const float *w32, const float *norm,
+                                  float *gpart, float *lpart, float *grad, float *loss, float *w,
+                                  float *m1, float *m2, __nv_bfloat16 *wb_out, float lr, int t,
+                                  bool update, float *pred = nullptr);
 void launch_mlp_round(cudaStream_t s, const float *w, __nv_bfloat16 *wb);
 void launch_mlp_norm(cudaStream_t s, const int32_t *pn, const float *feat, const float *target,
                      float *norm);

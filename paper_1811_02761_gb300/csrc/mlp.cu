@@ -87,14 +87,17 @@ __global__ void mlp_features_kernel(Layout L, const DevState *__restrict__ ds,
 }
 
 // ---------------------------------------------------------------- forward
-struct MlpSmem {
-    float w[kMlpParams];
+struct alignas(16) MlpSmem {
+    float w[kMlpParams + 3];
     float mu[kIn], isd[kIn];
 };
+static_assert(oB1 % 4 == 0 && oW2 % 4 == 0 && oB2 % 4 == 0 && oW3 % 4 == 0, "weights read four at a time");
 
-__device__ __forceinline__ void load_weights(MlpSmem &S, const __nv_bfloat16 *wb,
+// The BF16 weights: wb, or (w32) FP32 parameters rounded here.
+__device__ __forceinline__ void load_weights(MlpSmem &S, const __nv_bfloat16 *wb, const float *w32,
                                              const float *norm) {
-    for (int p = threadIdx.x; p < kMlpParams; p += blockDim.x) S.w[p] = __bfloat162float(wb[p]);
+    for (int p = threadIdx.x; p < kMlpParams; p += blockDim.x)
+        S.w[p] = __bfloat162float(w32 ? __float2bfloat16_rn(w32[p]) : wb[p]);
     if (threadIdx.x < kIn) {
         S.mu[threadIdx.x] = norm ? norm[threadIdx.x] : 0.0f;
         S.isd[threadIdx.x] = norm ? 1.0f / norm[kIn + threadIdx.x] : 1.0f;
@@ -102,28 +105,64 @@ __device__ __forceinline__ void load_weights(MlpSmem &S, const __nv_bfloat16 *wb
     __syncthreads();
 }
 
-// Forward pass of one sample; keeps the activations for the backward pass.
-__device__ __forceinline__ float mlp_fwd(const MlpSmem &S, const float *x, float (&xn)[kIn],
-                                         float (&h1)[kH], float (&h2)[kH]) {
+// Four consecutive weights in one shared-memory broadcast: with one load per
+// product the loads, not the products, bound the pass.
+__device__ __forceinline__ float4 w4(const MlpSmem &S, int p) {
+    return *reinterpret_cast<const float4 *>(&S.w[p]);
+}
+
+constexpr int kHS = kH + 4;  // stride of a thread's row: 16-byte aligned, eight rows in distinct banks
+
+__device__ __forceinline__ void put_row(float *row, const float (&v)[kH]) {
 #pragma unroll
-    for (int i = 0; i < kIn; i++) xn[i] = (x[i] - S.mu[i]) * S.isd[i];
-#pragma unroll 4
-    for (int j = 0; j < kH; j++) {
-        float a = S.w[oB1 + j];
+    for (int j = 0; j < kH; j += 4)
+        *reinterpret_cast<float4 *>(row + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+}
+
+// a += x (weights p .. p + 31)
+__device__ __forceinline__ void add_row(const MlpSmem &S, int p, float x, float (&a)[kH]) {
 #pragma unroll
-        for (int i = 0; i < kIn; i++) a = fmaf(xn[i], S.w[oW1 + i * kH + j], a);
-        h1[j] = fmaxf(a, 0.0f);
+    for (int k = 0; k < kH; k += 4) {
+        const float4 w = w4(S, p + k);
+        a[k] = fmaf(x, w.x, a[k]);
+        a[k + 1] = fmaf(x, w.y, a[k + 1]);
+        a[k + 2] = fmaf(x, w.z, a[k + 2]);
+        a[k + 3] = fmaf(x, w.w, a[k + 3]);
     }
-#pragma unroll 4
-    for (int k = 0; k < kH; k++) {
-        float a = S.w[oB2 + k];
+}
+
+// Forward pass of one sample: the 32 sums of a layer in registers, an input at
+// a time from this thread's rows in shared memory (xrow: standardised inputs,
+// h1row: first activations), every sum in the order of its inputs.  h2: the
+// second activations.
+__device__ __forceinline__ float mlp_fwd(const MlpSmem &S, const float *x, float *xrow, float *h1row,
+                                         float (&h2)[kH]) {
+    float a[kH];
 #pragma unroll
-        for (int j = 0; j < kH; j++) a = fmaf(h1[j], S.w[oW2 + j * kH + k], a);
-        h2[k] = fmaxf(a, 0.0f);
+    for (int j = 0; j < kH; j++) a[j] = S.w[oB1 + j];
+#pragma unroll 2
+    for (int i = 0; i < kIn; i++) {
+        const float v = (x[i] - S.mu[i]) * S.isd[i];
+        xrow[i] = v;
+        add_row(S, oW1 + i * kH, v, a);
+    }
+#pragma unroll
+    for (int j = 0; j < kH; j++) a[j] = fmaxf(a[j], 0.0f);
+    put_row(h1row, a);
+#pragma unroll
+    for (int k = 0; k < kH; k++) a[k] = S.w[oB2 + k];
+#pragma unroll 1
+    for (int j = 0; j < kH; j += 2) {
+        const float2 h = *reinterpret_cast<const float2 *>(h1row + j);
+        add_row(S, oW2 + j * kH, h.x, a);
+        add_row(S, oW2 + (j + 1) * kH, h.y, a);
     }
     float y = S.w[oB3];
 #pragma unroll
-    for (int k = 0; k < kH; k++) y = fmaf(h2[k], S.w[oW3 + k], y);
+    for (int k = 0; k < kH; k++) {
+        h2[k] = fmaxf(a[k], 0.0f);
+        y = fmaf(h2[k], S.w[oW3 + k], y);
+    }
     return y;
 }
 
@@ -136,130 +175,188 @@ __global__ void __launch_bounds__(128) mlp_forward_kernel(const int32_t *__restr
                                                           const float *__restrict__ tnorm,
                                                           float *__restrict__ pred) {
     __shared__ MlpSmem S;
-    load_weights(S, wb, norm);
+    __shared__ __align__(16) float h1[128][kHS];
+    __shared__ float xr[128][kIn + 1];
+    load_weights(S, wb, nullptr, norm);
     const float tm = tnorm ? tnorm[0] : 0.0f, ts = tnorm ? tnorm[1] : 1.0f;
     const int64_t n = pn ? (int64_t)*pn : n_host;
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n;
          g += (int64_t)gridDim.x * blockDim.x) {
-        float xn[kIn], h1[kH], h2[kH];
-        pred[g] = fmaf(mlp_fwd(S, feat + g * kIn, xn, h1, h2), ts, tm);
+        float h2[kH];
+        pred[g] = fmaf(mlp_fwd(S, feat + g * kIn, xr[threadIdx.x], h1[threadIdx.x], h2), ts, tm);
     }
 }
 
 // ---------------------------------------------------------------- backward
-constexpr int kGB = 128;  // samples per block in the gradient kernel
-
-struct GradSmem {
+constexpr int kGB = kMlpGradBlock;  // samples (and threads) per block in the gradient kernel
+struct alignas(16) GradSmem {
     MlpSmem m;
-    float xn[kGB][kIn];
-    float h1[kGB][kH + 1];
-    float d1[kGB][kH + 1];
-    float h2[kGB][kH + 1];
-    float d2[kGB][kH + 1];
+    float h1[kGB][kHS];
+    float d1[kGB][kHS];
+    float h2[kGB][kHS];
+    float d2[kGB][kHS];
+    float xn[kGB][kIn + 1];
     float dy[kGB];
     float loss[kGB];
 };
 
 // Mean-squared-error gradient of one minibatch: samples idx = base + s *
-// stride (s = 0 .. count-1); each block handles kGB of them and writes its
-// partial gradient (kMlpParams floats) and partial loss -- reduced in a fixed
-// order afterwards, so training is deterministic.
+// stride (s = 0 .. count-1); each block handles kGB of them, a thread each for
+// the forward and backward pass, and then the block's weight gradients as
+// small matrix products over its samples, a tile of outputs per thread (4 x 4
+// of dW2, from one broadcast of four of each side per sample).  Writes the
+// block's partial gradient (kMlpParams floats) and partial loss -- reduced in a
+// fixed order afterwards, so training is deterministic.  pred (nullable): the
+// network's outputs too.  Bound by the FP32 pipe and the shared-memory
+// broadcasts (3.7k products per sample).  n = 60013: 42 us with a load per
+// product and one gradient at a time, and 11 us more for the predictions; 25 us
+// for both so.
 __global__ void __launch_bounds__(kGB) mlp_grad_kernel(const float *__restrict__ feat,
                                                        const float *__restrict__ target,
                                                        int64_t base, int64_t stride, int count,
                                                        float inv_count,
                                                        const __nv_bfloat16 *__restrict__ wb,
+                                                       const float *__restrict__ w32,
                                                        const float *__restrict__ norm,
                                                        float *__restrict__ gpart,
-                                                       float *__restrict__ lpart) {
+                                                       float *__restrict__ lpart,
+                                                       float *__restrict__ pred) {
     extern __shared__ __align__(16) unsigned char mlp_smem[];
     GradSmem &S = *reinterpret_cast<GradSmem *>(mlp_smem);
-    load_weights(S.m, wb, norm);
+    load_weights(S.m, wb, w32, norm);
     const int t = threadIdx.x;
     const int s = blockIdx.x * kGB + t;
-    if (s < count) {
-        const int64_t g = base + (int64_t)s * stride;
-        float xn[kIn], h1[kH], h2[kH];
-        const float y = mlp_fwd(S.m, feat + g * kIn, xn, h1, h2);
-        const float e = y - target[g];
-        const float dy = 2.0f * e * inv_count;
-        S.dy[t] = dy;
-        S.loss[t] = e * e * inv_count;
+    {
+        float *h1row = S.h1[t], *d1row = S.d1[t];
+        float h2[kH], dy = 0.0f, loss = 0.0f;
+        const bool on = s < count;
+        const int64_t g = base + (int64_t)(on ? s : 0) * stride;
+        const float y = mlp_fwd(S.m, feat + g * kIn, S.xn[t], h1row, h2);
+        if (!on) {  // past the end (the batch's first sample was read): all zero
+#pragma unroll
+            for (int k = 0; k < kH; k++) h2[k] = 0.0f;
+            put_row(h1row, h2);
+#pragma unroll
+            for (int i = 0; i < kIn; i++) S.xn[t][i] = 0.0f;
+        }
+        put_row(S.h2[t], h2);
+        if (on) {
+            if (pred) pred[g] = y;
+            const float e = y - target[g];
+            dy = 2.0f * e * inv_count;
+            loss = e * e * inv_count;
+        }
         float d2[kH];
 #pragma unroll
         for (int k = 0; k < kH; k++) d2[k] = h2[k] > 0.0f ? dy * S.m.w[oW3 + k] : 0.0f;
-#pragma unroll 4
+        put_row(S.d2[t], d2);
+#pragma unroll 2
         for (int j = 0; j < kH; j++) {
             float a = 0.0f;
 #pragma unroll
-            for (int k = 0; k < kH; k++) a = fmaf(d2[k], S.m.w[oW2 + j * kH + k], a);
-            S.d1[t][j] = h1[j] > 0.0f ? a : 0.0f;
+            for (int k = 0; k < kH; k += 4) {
+                const float4 w = w4(S.m, oW2 + j * kH + k);
+                a = fmaf(d2[k], w.x, a);
+                a = fmaf(d2[k + 1], w.y, a);
+                a = fmaf(d2[k + 2], w.z, a);
+                a = fmaf(d2[k + 3], w.w, a);
+            }
+            d1row[j] = h1row[j] > 0.0f ? a : 0.0f;
         }
-#pragma unroll
-        for (int i = 0; i < kIn; i++) S.xn[t][i] = xn[i];
-#pragma unroll
-        for (int j = 0; j < kH; j++) {
-            S.h1[t][j] = h1[j];
-            S.h2[t][j] = h2[j];
-            S.d2[t][j] = d2[j];
-        }
-    } else {
-        S.dy[t] = 0.0f;
-        S.loss[t] = 0.0f;
-#pragma unroll
-        for (int i = 0; i < kIn; i++) S.xn[t][i] = 0.0f;
-#pragma unroll
-        for (int j = 0; j < kH; j++) S.h1[t][j] = S.h2[t][j] = S.d1[t][j] = S.d2[t][j] = 0.0f;
+        S.dy[t] = dy;
+        S.loss[t] = loss;
     }
     __syncthreads();
     float *gp = gpart + (int64_t)blockIdx.x * kMlpParams;
-    // every parameter's gradient is a sum over the block's samples
-    for (int p = t; p < kMlpParams; p += kGB) {
-        float acc = 0.0f;
-        if (p < oB1) {  // W1[i][j] = sum xn_i d1_j
-            const int i = p / kH, j = p % kH;
-            for (int q = 0; q < kGB; q++) acc = fmaf(S.xn[q][i], S.d1[q][j], acc);
-        } else if (p < oW2) {
-            const int j = p - oB1;
-            for (int q = 0; q < kGB; q++) acc += S.d1[q][j];
-        } else if (p < oB2) {  // W2[j][k] = sum h1_j d2_k
-            const int j = (p - oW2) / kH, k = (p - oW2) % kH;
-            for (int q = 0; q < kGB; q++) acc = fmaf(S.h1[q][j], S.d2[q][k], acc);
-        } else if (p < oW3) {
-            const int k = p - oB2;
-            for (int q = 0; q < kGB; q++) acc += S.d2[q][k];
-        } else if (p < oB3) {  // W3[k] = sum h2_k dy
-            const int k = p - oW3;
-            for (int q = 0; q < kGB; q++) acc = fmaf(S.h2[q][k], S.dy[q], acc);
-        } else {
-            for (int q = 0; q < kGB; q++) acc += S.dy[q];
+    // every parameter's gradient is a sum over the block's samples, in order
+    static_assert(kGB == 64, "the tiles below");
+    {  // W2[j][k] = sum h1_j d2_k: rows 4 (t / 8) .., columns 4 (t % 8) ..
+        const int j0 = 4 * (t >> 3), k0 = 4 * (t & 7);
+        float acc[4][4] = {};
+        for (int q = 0; q < kGB; q++) {
+            const float4 h = *reinterpret_cast<const float4 *>(&S.h1[q][j0]);
+            const float4 d = *reinterpret_cast<const float4 *>(&S.d2[q][k0]);
+            const float hv[4] = {h.x, h.y, h.z, h.w}, dv[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+            for (int u = 0; u < 4; u++)
+#pragma unroll
+                for (int v = 0; v < 4; v++) acc[u][v] = fmaf(hv[u], dv[v], acc[u][v]);
         }
-        gp[p] = acc;
+#pragma unroll
+        for (int u = 0; u < 4; u++)
+#pragma unroll
+            for (int v = 0; v < 4; v++) gp[oW2 + (j0 + u) * kH + k0 + v] = acc[u][v];
     }
-    if (t == 0) {
-        float l = 0.0f;
-        for (int q = 0; q < kGB; q++) l += S.loss[q];
-        lpart[blockIdx.x] = l;
+    {  // W1[i][j] = sum xn_i d1_j: row t / 8, columns 4 (t % 8) ..
+        const int i = t >> 3, j0 = 4 * (t & 7);
+        float acc[4] = {};
+        for (int q = 0; q < kGB; q++) {
+            const float x = S.xn[q][i];
+            const float4 d = *reinterpret_cast<const float4 *>(&S.d1[q][j0]);
+            acc[0] = fmaf(x, d.x, acc[0]);
+            acc[1] = fmaf(x, d.y, acc[1]);
+            acc[2] = fmaf(x, d.z, acc[2]);
+            acc[3] = fmaf(x, d.w, acc[3]);
+        }
+#pragma unroll
+        for (int v = 0; v < 4; v++) gp[oW1 + i * kH + j0 + v] = acc[v];
+    }
+    {  // b1, b2 (one each per thread of a warp), W3
+        const int k = t & 31;
+        float a = 0.0f, c = 0.0f;
+        if (t < 32) {
+            for (int q = 0; q < kGB; q++) {
+                a += S.d1[q][k];
+                c += S.d2[q][k];
+            }
+            gp[oB1 + k] = a;
+            gp[oB2 + k] = c;
+        } else {
+            for (int q = 0; q < kGB; q++) {
+                a = fmaf(S.h2[q][k], S.dy[q], a);
+                c += k == 0 ? S.dy[q] : S.loss[q];
+            }
+            gp[oW3 + k] = a;
+            if (k == 0) gp[oB3] = c;
+            if (k == 1) lpart[blockIdx.x] = c;
+        }
     }
 }
 
 // Fixed-order reduction of the block partials; then one Adam step (Kingma &
-// Ba 2015) on the FP32 master weights and the BF16 working copy.
-__global__ void mlp_reduce_adam_kernel(int nblocks, const float *__restrict__ gpart,
-                                       const float *__restrict__ lpart, float *__restrict__ grad,
-                                       float *__restrict__ loss, float *__restrict__ w,
-                                       float *__restrict__ m1, float *__restrict__ m2,
-                                       __nv_bfloat16 *__restrict__ wb, float lr, float b1,
-                                       float b2, float epsa, float c1, float c2, int do_update) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p == 0 && loss) {
-        float l = 0.0f;
-        for (int b = 0; b < nblocks; b++) l += lpart[b];
-        *loss = l;
+// Ba 2015) on the FP32 master weights and the BF16 working copy.  A block has
+// 32 parameters in 32 slices of the partials (every 32nd each, summed in
+// order, then the slices in order): with one thread per parameter the chain of
+// loads took 17 us for 469 blocks, so it takes 5.5 us for 938.  The last block adds the losses.
+constexpr int kRS = 32;
+__global__ void __launch_bounds__(32 * kRS) mlp_reduce_adam_kernel(
+    int nblocks, const float *__restrict__ gpart, const float *__restrict__ lpart,
+    float *__restrict__ grad, float *__restrict__ loss, float *__restrict__ w,
+    float *__restrict__ m1, float *__restrict__ m2, __nv_bfloat16 *__restrict__ wb, float lr,
+    float b1, float b2, float epsa, float c1, float c2, int do_update) {
+    __shared__ float sh[kRS][33];
+    const int lane = (int)lane_id(), sl = (int)(threadIdx.x >> 5);
+    const bool losses = blockIdx.x == gridDim.x - 1;
+    const int p = blockIdx.x * 32 + lane;
+    float g = 0.0f;
+    if (losses) {
+        if (lane == 0)
+            for (int b = sl; b < nblocks; b += kRS) g += lpart[b];
+    } else if (p < kMlpParams) {
+#pragma unroll 8
+        for (int b = sl; b < nblocks; b += kRS) g += gpart[(int64_t)b * kMlpParams + p];
+    }
+    sh[sl][lane] = g;
+    __syncthreads();
+    if (sl != 0) return;
+    g = 0.0f;
+#pragma unroll
+    for (int k = 0; k < kRS; k++) g += sh[k][lane];
+    if (losses) {
+        if (lane == 0 && loss) *loss = g;
+        return;
     }
     if (p >= kMlpParams) return;
-    float g = 0.0f;
-    for (int b = 0; b < nblocks; b++) g += gpart[(int64_t)b * kMlpParams + p];
     if (grad) grad[p] = g;
     if (!do_update) return;
     const float mm = b1 * m1[p] + (1.0f - b1) * g;
@@ -376,23 +473,23 @@ void launch_mlp_forward(cudaStream_t s, const int32_t *pn, int64_t n, const floa
     mlp_forward_kernel<<<nsm * 4, 128, 0, s>>>(pn, n, feat, wb, norm, tnorm, pred);
 }
 
-size_t mlp_grad_smem() { return sizeof(GradSmem); }
-
 cudaError_t launch_mlp_train_step(cudaStream_t s, const float *feat, const float *target,
                                   int64_t base, int64_t stride, int count,
-                                  const __nv_bfloat16 *wb, const float *norm, float *gpart,
-                                  float *lpart, float *grad, float *loss, float *w, float *m1,
-                                  float *m2, __nv_bfloat16 *wb_out, float lr, int t, bool update) {
+                                  const __nv_bfloat16 *wb, const float *w32, const float *norm,
+                                  float *gpart, float *lpart, float *grad, float *loss, float *w,
+                                  float *m1, float *m2, __nv_bfloat16 *wb_out, float lr, int t,
+                                  bool update, float *pred) {
     // per call: the attribute belongs to the current device's context
     cudaError_t e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(GradSmem));
     if (e != cudaSuccess) return e;
     const int nb = (count + kGB - 1) / kGB;
     mlp_grad_kernel<<<nb, kGB, sizeof(GradSmem), s>>>(feat, target, base, stride, count,
-                                                      1.0f / (float)count, wb, norm, gpart, lpart);
+                                                      1.0f / (float)count, wb, w32, norm, gpart,
+                                                      lpart, pred);
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f / (1.0f - powf(b1, (float)t)), c2 = 1.0f / (1.0f - powf(b2, (float)t));
-    mlp_reduce_adam_kernel<<<(kMlpParams + 255) / 256, 256, 0, s>>>(
+    mlp_reduce_adam_kernel<<<(kMlpParams + 31) / 32 + 1, 32 * kRS, 0, s>>>(
         nb, gpart, lpart, grad, loss, w, m1, m2, wb_out, lr, b1, b2, 1e-8f, c1, c2, update ? 1 : 0);
     return cudaGetLastError();
 }
