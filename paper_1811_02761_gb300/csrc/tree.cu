@@ -374,8 +374,8 @@ __device__ __forceinline__ void write_quad(int id, const float q[6], float4 *nod
 
 // One internal node per team of eight lanes from its children's records
 // (contiguous, at most 8), a lane per child; every lane of the warp calls this
-// (go false: a team without a node).  Sums are reduced over the team pairwise,
-// relative to the cell centre; the size is
+// (go false: a team without a node).  Sums run over the children in octant
+// order, relative to the cell centre; the size is
 //   b = min(max_c (|com_c - com| + b_c), distance from com to the farthest
 //           corner of the cell widened by one finest cell),
 // rounded up.  After a refit (positions moved since the build, members may
@@ -426,16 +426,24 @@ __device__ __forceinline__ bool internal_nodes(const Layout &L, bool go, int p, 
     }
     CellF cell{};
     if (ok) cell = node_cell(L, key, level, box);
+    // the sums over the children run in octant order in every lane (a lane
+    // without a child adds zeros), so they are those of one thread
     const float w = A.w;
-    float px = w * (A.x - cell.c[0]), py = w * (A.y - cell.c[1]), pz = w * (A.z - cell.c[2]);
+    const float ox = has ? A.x - cell.c[0] : 0.0f, oy = has ? A.y - cell.c[1] : 0.0f,
+                oz = has ? A.z - cell.c[2] : 0.0f;
+    const float2 mine = M;
+    const int cmine = count;
+    M = make_float2(0.0f, 0.0f);
+    count = 0;
+    float px = 0.0f, py = 0.0f, pz = 0.0f;
 #pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-        const float2 Mo = make_float2(__shfl_xor_sync(NB_FULL, M.x, o), __shfl_xor_sync(NB_FULL, M.y, o));
-        M = df_add(M, Mo);
-        px += __shfl_xor_sync(NB_FULL, px, o);
-        py += __shfl_xor_sync(NB_FULL, py, o);
-        pz += __shfl_xor_sync(NB_FULL, pz, o);
-        count += __shfl_xor_sync(NB_FULL, count, o);
+    for (int k = 0; k < 8; k++) {
+        const float wk = __shfl_sync(NB_FULL, w, k, 8);
+        M = df_add(M, make_float2(__shfl_sync(NB_FULL, mine.x, k, 8), __shfl_sync(NB_FULL, mine.y, k, 8)));
+        px = fmaf(wk, __shfl_sync(NB_FULL, ox, k, 8), px);
+        py = fmaf(wk, __shfl_sync(NB_FULL, oy, k, 8), py);
+        pz = fmaf(wk, __shfl_sync(NB_FULL, oz, k, 8), pz);
+        count += __shfl_sync(NB_FULL, cmine, k, 8);
     }
     float cp[3] = {cell.c[0], cell.c[1], cell.c[2]};
     if (M.x > 0.0f) {
@@ -447,13 +455,18 @@ __device__ __forceinline__ bool internal_nodes(const Layout &L, bool go, int p, 
     float rec = has ? __fadd_ru(__fsqrt_ru(r2), b) : 0.0f;
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) rec = fmaxf(rec, __shfl_xor_sync(NB_FULL, rec, o));
-    float q[6] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y};
+    float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (nodeQ) {
-        if (has) quad_add(q, w, dx, dy, dz, r2);
+        const float qm[6] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y};
 #pragma unroll
-        for (int o = 1; o < 8; o <<= 1)
+        for (int k = 0; k < 8; k++) {
 #pragma unroll
-            for (int k = 0; k < 6; k++) q[k] += __shfl_xor_sync(NB_FULL, q[k], o);
+            for (int a = 0; a < 6; a++) q[a] += __shfl_sync(NB_FULL, qm[a], k, 8);
+            quad_add(q, __shfl_sync(NB_FULL, w, k, 8), __shfl_sync(NB_FULL, has ? dx : 0.0f, k, 8),
+                     __shfl_sync(NB_FULL, has ? dy : 0.0f, k, 8),
+                     __shfl_sync(NB_FULL, has ? dz : 0.0f, k, 8),
+                     __shfl_sync(NB_FULL, has ? r2 : 0.0f, k, 8));
+        }
     }
     if (ok && sub == 0) {
         float c2 = 0.0f;
@@ -471,13 +484,14 @@ __device__ __forceinline__ bool internal_nodes(const Layout &L, bool go, int p, 
     return ok || !go;
 }
 
-// Count a finished node in at its parent `par` (one atomic add with release
-// and acquire semantics: this thread's writes of the node are published by
-// it, and the thread that completes the parent sees every child's records).
-// Returns how many of the parent's children have now arrived.
+// Count a finished node in at its parent `par`; the caller has fenced the
+// node's records before, and the lane that completes the parent fences after
+// it, so it sees every child's records.  (A relaxed add between the two fences:
+// an add with release and acquire semantics would fence a second time on every
+// level of the climb.)  Returns how many of the parent's children have arrived.
 __device__ __forceinline__ int count_in(int par, int32_t *node_arrive) {
     int old;
-    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
+    asm volatile("atom.relaxed.gpu.global.add.s32 %0, [%1], 1;"
                  : "=r"(old)
                  : "l"(node_arrive + par)
                  : "memory");
@@ -611,12 +625,11 @@ __global__ void __launch_bounds__(256, NB_MOMENTS_MIN_CTAS) moments_kernel(
             }
         }
         // internal nodes: the chunk's leaf records are device-visible before
-        // any lane counts a leaf in (the writers' fence, then the warp
-        // barrier).  A climbing thread carries a member key (its leaf's first
+        // any lane counts a leaf in (the warp barrier, then the lane's fence).  A climbing thread carries a member key (its leaf's first
         // particle): every ancestor's cell follows from it and the ancestor's
         // level, one up per step.
-        __threadfence();
         __syncwarp();
+        __threadfence();
         int node = id0, par = -1, level = 0;
         uint64_t key = 0;
         if (leaf) {
@@ -639,6 +652,7 @@ __global__ void __launch_bounds__(256, NB_MOMENTS_MIN_CTAS) moments_kernel(
                     ready = count_in(par, node_arrive) == nc;
                 }
             }
+            if (ready) __threadfence();
             unsigned rm = __ballot_sync(NB_FULL, ready);
             if (!rm) break;
             while (rm) {  // four parents at a time, eight lanes each
@@ -659,8 +673,8 @@ __global__ void __launch_bounds__(256, NB_MOMENTS_MIN_CTAS) moments_kernel(
                     bad = true;  // still counted in above, so the counters stay consistent
             }
             // the teams' records are device-visible before any lane counts one in
-            __threadfence();
             __syncwarp();
+            __threadfence();
             if (ready) {
                 node_arrive[par] = 0;
                 node = par;
