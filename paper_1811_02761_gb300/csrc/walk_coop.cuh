@@ -59,7 +59,7 @@ __host__ __device__ inline size_t coop_smem(int list_depth, int stack_depth, boo
 }
 
 template <int IPL, bool PHI, bool COMP, bool SAFE, bool QUAD>
-__global__ void __maxnreg__(walk_regs<IPL>())
+__global__ void __maxnreg__((walk_regs<IPL, QUAD || COMP>()))
     coop_walk_kernel(WalkArgs a, int geometric, int second) {
     constexpr int W = kCoopWarps;
     extern __shared__ __align__(16) unsigned char walk_smem[];

@@ -463,6 +463,11 @@ __device__ __forceinline__ bool over_quota(const WalkArgs &a, int entries, int n
 // Register budget of the walk kernel per thread: 64 (32 resident warps per
 // SM) while a lane holds at most two i-particles; more slots need more
 // registers for the positions and sums they keep (build-time tunable).
+// Quadrupoles and compensated sums (MORE) keep more still: at three slots they
+// spilled up to 1.3 KB at 80 registers, and 16 warps per SM without spills beat
+// 24 with them (galaxy 300007, quadrupoles, 2^-12: 1.60 -> 1.53 ms, 96
+// registers 1.52; Plummer 4096 with quadrupoles, cooperative, 67 -> 57 us;
+// compensated, 300000 at 2^-20, 9.5 -> 9.1 ms).
 #ifndef NB_WALK_REGS_2
 #define NB_WALK_REGS_2 64
 #endif
@@ -472,13 +477,14 @@ __device__ __forceinline__ bool over_quota(const WalkArgs &a, int entries, int n
 #ifndef NB_WALK_REGS_4
 #define NB_WALK_REGS_4 96
 #endif
-template <int IPL>
+template <int IPL, bool MORE>
 constexpr int walk_regs() {
+    if (MORE && IPL >= 3) return 128;
     return IPL <= 2 ? NB_WALK_REGS_2 : (IPL == 3 ? NB_WALK_REGS_3 : NB_WALK_REGS_4);
 }
 
 template <int IPL, bool PHI, bool COMP, bool SAFE, bool QUAD>
-__global__ void __maxnreg__(walk_regs<IPL>()) walk_kernel(WalkArgs a, int geometric) {
+__global__ void __maxnreg__((walk_regs<IPL, QUAD || COMP>())) walk_kernel(WalkArgs a, int geometric) {
     extern __shared__ __align__(16) unsigned char walk_smem[];
     const int D = a.list_depth, S = a.stack_depth;
     const int DQ = QUAD ? walk_quad_depth(D) : 0;
