@@ -92,6 +92,9 @@ struct nbody_ctx {
     // staging of host arrays
     DevBuf stage[12];
     double *h_diag = nullptr;  // pinned
+    char *h_sys = nullptr;     // pinned: offsets, eps, eps^2 on their way to the device
+    size_t h_sys_bytes = 0;
+    cudaEvent_t sys_ev = nullptr;
 
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
     std::vector<cudaEvent_t> wev;  // (start, end) pairs around walk-kernel launches
@@ -469,28 +472,37 @@ nbody_status refit_tree_groups(nbody_ctx *c, const Layout &L, const float *aold 
     return NBODY_OK;
 }
 
-// Upload the CSR offsets and per-system eps^2.
+// Upload the CSR offsets, per-system eps and eps^2, from page-locked memory:
+// the copies are ordered before the call's kernels and need no wait (from
+// pageable memory they cost three staged copies and a synchronisation, about
+// 25 us of every call).
 nbody_status upload_systems(nbody_ctx *c, int nsys, const int64_t *offsets, const float *eps_sys) {
-    std::vector<int64_t> off(nsys + 1);
-    std::vector<float> e2(nsys), e1(nsys);
-    if (offsets) {
-        std::memcpy(off.data(), offsets, sizeof(int64_t) * (nsys + 1));
-    } else {
-        off[0] = 0;
+    const size_t ob = sizeof(int64_t) * (size_t)(nsys + 1), eb = sizeof(float) * (size_t)nsys;
+    if (!c->sys_ev) NB_CUDA(c, cudaEventCreateWithFlags(&c->sys_ev, cudaEventDisableTiming));
+    NB_CUDA(c, cudaEventSynchronize(c->sys_ev));  // an earlier call's copies (all but always done)
+    if (c->h_sys_bytes < ob + 2 * eb) {
+        if (c->h_sys) cudaFreeHost(c->h_sys);
+        c->h_sys = nullptr;
+        c->h_sys_bytes = 0;
+        if (cudaMallocHost(&c->h_sys, ob + 2 * eb) != cudaSuccess) {
+            cudaGetLastError();
+            c->h_sys = nullptr;
+            return fail(c, NBODY_ENOMEM, "host allocation");
+        }
+        c->h_sys_bytes = ob + 2 * eb;
     }
+    int64_t *off = reinterpret_cast<int64_t *>(c->h_sys);
+    float *e1 = reinterpret_cast<float *>(c->h_sys + ob), *e2 = e1 + nsys;
+    std::memcpy(off, offsets, ob);
     for (int s = 0; s < nsys; s++) {
-        float e = eps_sys ? eps_sys[s] : c->cfg.eps;
+        const float e = eps_sys ? eps_sys[s] : c->cfg.eps;
         e1[s] = e;
         e2[s] = e * e;
     }
-    NB_CUDA(c, cudaMemcpyAsync(c->sys_off.p, off.data(), sizeof(int64_t) * (nsys + 1),
-                               cudaMemcpyHostToDevice, c->stream));
-    NB_CUDA(c, cudaMemcpyAsync(c->sys_eps2.p, e2.data(), sizeof(float) * nsys,
-                               cudaMemcpyHostToDevice, c->stream));
-    NB_CUDA(c, cudaMemcpyAsync(c->sys_eps.p, e1.data(), sizeof(float) * nsys,
-                               cudaMemcpyHostToDevice, c->stream));
-    // the copies read pageable host vectors: make sure they have completed
-    NB_CUDA(c, cudaStreamSynchronize(c->stream));
+    NB_CUDA(c, cudaMemcpyAsync(c->sys_off.p, off, ob, cudaMemcpyHostToDevice, c->stream));
+    NB_CUDA(c, cudaMemcpyAsync(c->sys_eps2.p, e2, eb, cudaMemcpyHostToDevice, c->stream));
+    NB_CUDA(c, cudaMemcpyAsync(c->sys_eps.p, e1, eb, cudaMemcpyHostToDevice, c->stream));
+    NB_CUDA(c, cudaEventRecord(c->sys_ev, c->stream));
     return NBODY_OK;
 }
 
@@ -917,6 +929,8 @@ nbody_status nbody_destroy(nbody_ctx *ctx) {
     if (ctx->ds) cudaFree(ctx->ds);
     if (ctx->h_ds) cudaFreeHost(ctx->h_ds);
     if (ctx->h_diag) cudaFreeHost(ctx->h_diag);
+    if (ctx->h_sys) cudaFreeHost(ctx->h_sys);
+    if (ctx->sys_ev) cudaEventDestroy(ctx->sys_ev);
     for (auto &ev : ctx->ev)
         if (ev) cudaEventDestroy(ev);
     for (auto ev : ctx->wev) cudaEventDestroy(ev);
@@ -1202,9 +1216,10 @@ static nbody_status block_steps(nbody_ctx *ctx, const Layout &L, StepState *S, i
         if (st != NBODY_OK) return st;
         NB_CUDA(ctx, pool_event(ctx, &e1));
         NB_CUDA(ctx, cudaEventRecord(e1, q));
-        NB_CUDA(ctx, cudaMemcpyAsync(ctx->aold_s.p, S[cur].aold, (size_t)n * 4,
-                                     cudaMemcpyDeviceToDevice, q));
-        NB_CUDA(ctx, cudaMemsetAsync(dact, 0, sizeof(int32_t), q));
+        if (T == total)  // for the cost model's features after the call
+            NB_CUDA(ctx, cudaMemcpyAsync(ctx->aold_s.p, S[cur].aold, (size_t)n * 4,
+                                         cudaMemcpyDeviceToDevice, q));
+        // (the group pass has cleared both counts)
         launch_block_active_groups(q, ctx->ds, P<int32_t>(ctx->grp_first), P<int32_t>(ctx->grp_count),
                                    S[cur].lvl, T, K, P<int32_t>(ctx->grp_order), dact, ctx->nsm);
         ctx->kernels += 1;
@@ -1214,7 +1229,6 @@ static nbody_status block_steps(nbody_ctx *ctx, const Layout &L, StepState *S, i
         NB_CUDA(ctx, pool_event(ctx, &e2));
         NB_CUDA(ctx, cudaEventRecord(e2, q));
         marks.push_back(ctx->evused - 3);
-        NB_CUDA(ctx, cudaMemsetAsync(dmax, 0, sizeof(int32_t), q));
         launch_block_kick(q, n, S[cur], acc, T, total, dt, K, eta, P<int64_t>(ctx->sys_off), L.nsys,
                           P<float>(ctx->sys_eps), dmax);
         ctx->kernels += 1;

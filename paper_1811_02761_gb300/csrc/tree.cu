@@ -981,8 +981,9 @@ __global__ void __launch_bounds__(FL_T) flag_one_kernel(uint8_t *__restrict__ f,
 }
 
 // Warp per group: count, bounding-box centre and enclosing radius, system;
-// with aold also alpha (as group_alpha_kernel), and with queue the walk's
-// queues are reset: a step's walk then needs no launch of its own for either.
+// with aold also alpha (as group_alpha_kernel), and with reset the walk's
+// queues and a block step's counts are cleared: a step's walk then needs no
+// launch of its own for any of them.
 __global__ void __launch_bounds__(256) group_info_kernel(Layout L, int G,
                                                          const float4 *__restrict__ pos4,
                                                          const int64_t *__restrict__ off,
@@ -991,8 +992,11 @@ __global__ void __launch_bounds__(256) group_info_kernel(Layout L, int G,
                                                          int32_t *grp_count, float4 *grp_sphere,
                                                          int32_t *grp_sys,
                                                          const float *__restrict__ aold, float dacc,
-                                                         float *grp_alpha, WalkQueue *queue) {
-    if (queue && blockIdx.x == 0 && threadIdx.x == 0) *queue = WalkQueue{};
+                                                         float *grp_alpha, DevState *reset) {
+    if (reset && blockIdx.x == 0 && threadIdx.x == 0) {
+        reset->queue = WalkQueue{};
+        reset->block_maxlvl = reset->block_nactive = 0;  // of a block step's tick
+    }
     // a half-warp per group, two groups per warp at a time: both groups'
     // member loads are in flight together (min, max and the largest distance
     // do not depend on the order of the reduction)
@@ -1081,7 +1085,7 @@ void refit_groups(cudaStream_t s, const Layout &L, int group_size, const float4 
     if (gb > nsm * NB_GROUP_CTAS_PER_SM) gb = nsm * NB_GROUP_CTAS_PER_SM;
     group_info_kernel<<<gb, 256, 0, s>>>(L, group_size, pos4, d_off, ds, grp_first, grp_count,
                                          grp_sphere, grp_sys, aold, dacc, grp_alpha,
-                                         aold ? &ds->queue : nullptr);
+                                         aold ? ds : nullptr);
 }
 
 // alpha_g = delta_acc * min over members of |a_old| (Eq. 2 per group).

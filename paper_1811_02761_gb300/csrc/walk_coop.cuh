@@ -420,11 +420,18 @@ cudaError_t launch_coop_ipl(cudaStream_t s, const WalkArgs &a, const WalkShape &
         if (sh.compensated) k = sh.safe ? coop_walk_kernel<IPL, false, true, true, QUAD> : coop_walk_kernel<IPL, false, true, false, QUAD>;
         else k = sh.safe ? coop_walk_kernel<IPL, false, false, true, QUAD> : coop_walk_kernel<IPL, false, false, false, QUAD>;
     }
-    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = cudaSuccess;
+    if (smem > 48 * 1024) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-    int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, 32 * kCoopWarps, smem);
-    if (err != cudaSuccess) return err;
+    // resident CTAs, from the register and shared-memory budgets (no CTA waits
+    // for another, so a grid larger than that would only queue); an occupancy
+    // query on every launch costs more host time than the launch
+    constexpr int by_regs = 65536 / (32 * kCoopWarps * walk_regs<IPL, QUAD>());
+    const int more = 65536 / (32 * kCoopWarps * walk_regs<IPL, true>());
+    int per_sm = sh.compensated ? more : by_regs;
+    per_sm = per_sm > kCoopTarget ? kCoopTarget : per_sm;
+    const int by_smem = (int)(227 * 1024 / (smem + 1024));
+    if (per_sm > by_smem) per_sm = by_smem;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     if (sh.warps_launched && sh.coop_only) *sh.warps_launched = nsm * per_sm * kCoopWarps;
     k<<<nsm * per_sm, 32 * kCoopWarps, smem, s>>>(a, sh.geometric ? 1 : 0, 0);
