@@ -376,14 +376,14 @@ nbody_status build_core(nbody_ctx *c, const Layout &L, const void *x, const void
     c->kernels += bbox_kernels(L.nsys);
     if (L.n <= kRankSortMax) {
         launch_keys(s, L, x, y, z, dbl, P<int64_t>(c->sys_off), P<SysBox>(c->sys_box),
-                    P<uint64_t>(c->keys), P<uint32_t>(c->vals), nullptr, c->nsm);
+                    P<uint64_t>(c->keys), nullptr, nullptr, c->nsm);
         NB_CUDA(c, rank_sort(s, P<uint64_t>(c->keys), L.n, P<uint64_t>(c->keys_alt), P<uint32_t>(c->vals_alt)));
         c->kernels += 2;
         std::swap(c->keys, c->keys_alt);
         std::swap(c->vals, c->vals_alt);
     } else if (near_order && nosort_fits(L.n)) {
         launch_keys(s, L, x, y, z, dbl, P<int64_t>(c->sys_off), P<SysBox>(c->sys_box),
-                    P<uint64_t>(c->keys), P<uint32_t>(c->vals), nullptr, c->nsm);
+                    P<uint64_t>(c->keys), nullptr, nullptr, c->nsm);
         nosort(s, P<uint64_t>(c->keys), P<uint64_t>(c->keys_alt), P<uint32_t>(c->vals),
                P<uint32_t>(c->vals_alt), L.n, c->rs_temp.p, &c->ds->status);
         c->kernels += 1 + nosort_kernels();
@@ -391,7 +391,7 @@ nbody_status build_core(nbody_ctx *c, const Layout &L, const void *x, const void
         std::swap(c->vals, c->vals_alt);
     } else if (hint && nosort_fits(L.n)) {
         launch_keys(s, L, x, y, z, dbl, P<int64_t>(c->sys_off), P<SysBox>(c->sys_box),
-                    P<uint64_t>(c->keys), P<uint32_t>(c->vals), nullptr, c->nsm);
+                    P<uint64_t>(c->keys), nullptr, nullptr, c->nsm);
         nosort_hint_gather(s, L.n, P<uint64_t>(c->keys), hint, P<uint64_t>(c->keys_alt),
                            P<uint32_t>(c->vals_alt));
         // values: the caller indices; vals_alt is read by the scatter before

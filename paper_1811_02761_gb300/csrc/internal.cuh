@@ -153,7 +153,7 @@ void launch_bbox(cudaStream_t s, const Layout &L, const void *x, const void *y, 
 // empty, and *d_done zero).
 void launch_bbox_init(cudaStream_t s, int nsys, uint32_t *d_boxord);
 int bbox_kernels(int nsys);
-// Morton keys (vals = 0..n-1).  With sort_temp (cleared by radix_prepare),
+// Morton keys (vals, nullable: 0..n-1).  With sort_temp (cleared by radix_prepare),
 // the kernel also accumulates the radix sort's digit histograms, and the
 // sort is then called with hist_done = true.
 void launch_keys(cudaStream_t s, const Layout &L, const void *x, const void *y, const void *z,

@@ -82,14 +82,27 @@ __global__ void __launch_bounds__(256) bbox_kernel(int64_t n, const T *__restric
             }
         } else {
             for (int k = 0; k < 8; k++) {
-                int64_t i = base + k * 32 + lane;
-                if (i < n) {
-                    int s = sys_of(off, nsys, i);
+                // 32 particles of a chunk with several systems: one set of
+                // atomics per system among them, by its first lane
+                const int64_t i = base + k * 32 + lane;
+                const int s = i < n ? sys_of(off, nsys, i) : -1;
+                uint32_t v[3] = {0u, 0u, 0u};
+                if (i < n)
+                    for (int a = 0; a < 3; a++) v[a] = f2ord((float)p[a][i]);
+                unsigned todo = __ballot_sync(NB_FULL, s >= 0);
+                while (todo) {
+                    const int lead = __ffs(todo) - 1;
+                    const int ls = __shfl_sync(NB_FULL, s, lead);
+                    const unsigned same = __ballot_sync(NB_FULL, s == ls);
                     for (int a = 0; a < 3; a++) {
-                        uint32_t v = f2ord((float)p[a][i]);
-                        atomicMin(&boxord[s * 6 + a], v);
-                        atomicMax(&boxord[s * 6 + 3 + a], v);
+                        const uint32_t l = __reduce_min_sync(NB_FULL, s == ls ? v[a] : 0xffffffffu);
+                        const uint32_t h = __reduce_max_sync(NB_FULL, s == ls ? v[a] : 0u);
+                        if ((int)lane == lead) {
+                            atomicMin(&boxord[ls * 6 + a], l);
+                            atomicMax(&boxord[ls * 6 + 3 + a], h);
+                        }
                     }
+                    todo &= ~same;
                 }
             }
         }
@@ -108,27 +121,20 @@ __global__ void __launch_bounds__(256) bbox_kernel(int64_t n, const T *__restric
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const int nw = blockDim.x >> 5;
-        for (int q = 0; q < nw; q++) {
-            int s = sh_s[q];
-            if (s < 0) continue;
-            float l3[3], h3[3];
+    if (threadIdx.x < blockDim.x >> 5) {  // a thread per warp's record: the first of a system merges it
+        const int q = (int)threadIdx.x, nw = (int)(blockDim.x >> 5), s = sh_s[q];
+        bool mine = s >= 0;
+        for (int r = 0; r < q; r++) mine = mine && sh_s[r] != s;
+        if (mine) {
             for (int a = 0; a < 3; a++) {
-                l3[a] = sh_lo[q][a];
-                h3[a] = sh_hi[q][a];
-            }
-            for (int r = q + 1; r < nw; r++)
-                if (sh_s[r] == s) {
-                    for (int a = 0; a < 3; a++) {
-                        l3[a] = fminf(l3[a], sh_lo[r][a]);
-                        h3[a] = fmaxf(h3[a], sh_hi[r][a]);
+                float l = sh_lo[q][a], h = sh_hi[q][a];
+                for (int r = q + 1; r < nw; r++)
+                    if (sh_s[r] == s) {
+                        l = fminf(l, sh_lo[r][a]);
+                        h = fmaxf(h, sh_hi[r][a]);
                     }
-                    sh_s[r] = -1;
-                }
-            for (int a = 0; a < 3; a++) {
-                atomicMin(&boxord[s * 6 + a], f2ord(l3[a]));
-                atomicMax(&boxord[s * 6 + 3 + a], f2ord(h3[a]));
+                atomicMin(&boxord[s * 6 + a], f2ord(l));
+                atomicMax(&boxord[s * 6 + 3 + a], f2ord(h));
             }
         }
     }
@@ -467,7 +473,7 @@ __global__ void __launch_bounds__(256) keys_kernel(Layout L, const T *__restrict
             k = (spread3(qx) << 2) | (spread3(qy) << 1) | spread3(qz);
             if (L.sysbits) k |= (uint64_t)s << mbits;
             keys[i] = k;
-            vals[i] = (uint32_t)i;
+            if (vals) vals[i] = (uint32_t)i;
         }
         if (hist) hist_add(h, k, i < L.n, passes);
     }
