@@ -48,9 +48,9 @@ FP32_LANES_PER_SM = 128
 # warm-up-step walk, per particle; at another N the launch is scaled by
 # particles.  It is reported only while the walk source is the one the
 # counters were taken on (sha256 of walk_impl.cuh).
-WALK_TRAFFIC = {"bytes_per_particle": (230.617e6 + 110.988e6) / 8388608,
+WALK_TRAFFIC = {"bytes_per_particle": (230.606e6 + 110.991e6) / 8388608,
                 "n_captured": 8388608,
-                "walk_impl_sha256": "f45061adc710b78f6f6a1da075f2fc1840aeb28aed1bfb5370e2eeb20542bb67",
+                "walk_impl_sha256": "fb4f6dabbe23e1048edea65aeb64b61204e5fa5d06dd3ebbe89c8a98bba97f80",
                 "capture": "profiles/walk_kernel_traffic_galaxy_2e23.md"}
 
 
