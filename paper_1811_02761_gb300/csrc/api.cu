@@ -41,6 +41,7 @@ struct GraphKey {
     bool safe;
     bool mlp_norm;  // the cost model's input statistics were set at capture
     nbody_config cfg;
+    int64_t growths;  // buffers may move, and only some of them, when one grows
     const void *bufs[9];
 };
 
@@ -109,6 +110,7 @@ struct nbody_ctx {
     cudaStream_t gstream = nullptr;
     cudaGraphExec_t gexec = nullptr;
     GraphKey gkey{};
+    int64_t growths = 0;  // times that a buffer a graph may name was allocated anew
     int64_t gkernels = 0;
     bool capturing = false;  // enqueueing into a graph: no timing events
     int walk_warps = 0;      // resident warps of the last walk launch
@@ -305,6 +307,7 @@ cudaError_t ensure_capacity(nbody_ctx *c, int64_t n, int nsys, int levels) {
     cudaError_t e;
 #define NB_E(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
     if (n > c->cap_n) {
+        c->growths++;
         NB_E(ensure(c->keys, n * 8)); NB_E(ensure(c->keys_alt, n * 8));
         NB_E(ensure(c->vals, n * 4)); NB_E(ensure(c->vals_alt, n * 4));
         NB_E(ensure(c->pos4, n * 16)); NB_E(ensure(c->delta, n + 1)); NB_E(ensure(c->leaflev, n));
@@ -322,6 +325,7 @@ cudaError_t ensure_capacity(nbody_ctx *c, int64_t n, int nsys, int levels) {
     }
     int64_t cn = node_capacity(n, levels, c->cfg.leaf_cap, nsys);
     if (cn > c->cap_nodes) {
+        c->growths++;
         NB_E(ensure(c->node_start, cn * 4)); NB_E(ensure(c->node_level, cn));
         NB_E(ensure(c->node_parent, cn * 4)); NB_E(ensure(c->node_link, cn * 4));
         NB_E(ensure(c->node_count, cn * 4)); NB_E(ensure(c->node_nchild, cn * 4));
@@ -331,6 +335,7 @@ cudaError_t ensure_capacity(nbody_ctx *c, int64_t n, int nsys, int levels) {
         c->cap_nodes = cn;
     }
     if (nsys > c->cap_sys) {
+        c->growths++;
         NB_E(ensure(c->sys_off, (size_t)(nsys + 1) * 8)); NB_E(ensure(c->sys_box, (size_t)nsys * sizeof(SysBox)));
         NB_E(ensure(c->sys_boxord, (size_t)nsys * 24 + 4)); NB_E(ensure(c->sys_eps2, (size_t)nsys * 4));
         NB_E(ensure(c->sys_eps, (size_t)nsys * 4));
@@ -546,6 +551,7 @@ nbody_status do_build(nbody_ctx *c, int64_t n, int nsys, const int64_t *offsets,
                       const float *eps_sys, const float *x, const float *y, const float *z,
                       const float *m) {
     Layout L = make_layout(n, nsys);
+    c->aold_cur = nullptr;  // of the groups this build replaces
     cudaError_t e = ensure_capacity(c, n, nsys, L.levels);
     if (e != cudaSuccess) return fail(c, NBODY_ENOMEM, std::string("allocation: ") + cudaGetErrorString(e));
     std::vector<int64_t> off1 = {0, n};
@@ -639,8 +645,11 @@ cudaError_t ensure_coop(nbody_ctx *c) {
         if (e == cudaSuccess)
             e = cudaMemsetAsync(P<int32_t>(c->part_ctl) + kCutTasks, 0, (size_t)kCutTasks * 2 * 4, c->stream);
     }
-    if (e == cudaSuccess && c->L.n > kCoopParticles)
-        e = ensure(c->heavy, (size_t)heavy_records(c) * kHeavyWords * 4);
+    if (e == cudaSuccess && c->L.n > kCoopParticles) {
+        const size_t bytes = (size_t)heavy_records(c) * kHeavyWords * 4;
+        if (c->heavy.bytes < bytes) c->growths++;
+        e = ensure(c->heavy, bytes);
+    }
     return e;
 }
 
@@ -1253,9 +1262,11 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
     if (nsteps < 0) return fail(ctx, NBODY_EINVAL, "nsteps must be >= 0");
     if (!std::isfinite(dt)) return fail(ctx, NBODY_EINVAL, "dt must be finite");
     ctx->built = false;
+    ctx->aold_cur = nullptr;  // the state it points to may move
     cudaStream_t s = ctx->stream;
     Layout L = make_layout(n, nsys);
     cudaError_t e = ensure_capacity(ctx, n, nsys, L.levels);
+    if (ctx->st_buf[0][0].bytes < (size_t)n * 8) ctx->growths++;
     for (int b = 0; b < 2 && e == cudaSuccess; b++) {
         for (int k = 0; k < 3 && e == cudaSuccess; k++) e = ensure(ctx->st_buf[b][k], (size_t)n * 8);
         for (int k = 3; k < 10 && e == cudaSuccess; k++) e = ensure(ctx->st_buf[b][k], (size_t)n * 4);
@@ -1268,7 +1279,6 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
     if (st != NBODY_OK) return st;
     const bool safe = any_zero_eps(ctx, nsys, eps_sys);
     ctx->L = L;  // the walk's bounds checks read the particle count from here
-    ctx->aold_cur = nullptr;
     StepState S[2];
     for (int b = 0; b < 2; b++) {
         S[b].x = P<double>(ctx->st_buf[b][0]);
@@ -1433,6 +1443,7 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
         key.bufs[6] = ctx->pos4.p;
         key.bufs[7] = ctx->acc_s.p;
         key.bufs[8] = ctx->heavy.p;
+        key.growths = ctx->growths;
         if (!ctx->gstream)
             NB_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->gstream, cudaStreamNonBlocking));
         if (!ctx->gexec || std::memcmp(&key, &ctx->gkey, sizeof key) != 0) {
@@ -1923,25 +1934,27 @@ nbody_status nbody_mlp_eval(int64_t n, const float *features, const float *targe
     cudaStream_t s = (cudaStream_t)cuda_stream;
     const int nb = (int)((n + kMlpGradBlock - 1) / kMlpGradBlock);
     const size_t fsz = (size_t)n * 8 * 4, tsz = (size_t)n * 4, psz = kMlpParams * 4;
-    // Device arrays are read and written in place.  Host inputs are staged
+    // Arrays of the current device are read and written in place.  Others are staged
     // behind the partial sums; host outputs are written by the kernels into
     // page-locked memory and copied from there (three copies into pageable
     // memory took 100 us at n = 60013, allocating and freeing the device block
     // another 100).
     auto align = [](size_t v) { return (v + 255) & ~(size_t)255; };
     size_t dev = align((size_t)nb * psz) + align((size_t)nb * 4), host = 0;
+    int dev_id = 0;
+    if (cudaGetDevice(&dev_id) != cudaSuccess) return fail(nullptr, NBODY_ECUDA, "no device");
     const void *in[4] = {features, targets, params, norm};
     const size_t isz[4] = {fsz, tsz, psz, 64};
     size_t ioff[4];
     for (int k = 0; k < 4; k++) {
-        ioff[k] = in[k] && !is_device_ptr(in[k]) ? dev : SIZE_MAX;
+        ioff[k] = in[k] && !on_device(in[k], dev_id) ? dev : SIZE_MAX;
         if (ioff[k] != SIZE_MAX) dev += align(isz[k]);
     }
     void *out[3] = {pred, grad, loss};
     const size_t osz[3] = {tsz, psz, 4};
     size_t ooff[3];
     for (int k = 0; k < 3; k++) {
-        ooff[k] = out[k] && !is_device_ptr(out[k]) ? host : SIZE_MAX;
+        ooff[k] = out[k] && !on_device(out[k], dev_id) ? host : SIZE_MAX;
         if (ooff[k] != SIZE_MAX) host += align(osz[k]);
     }
     nb::Scratch scratch(s);
@@ -1954,7 +1967,7 @@ nbody_status nbody_mlp_eval(int64_t n, const float *features, const float *targe
         din[k] = static_cast<const float *>(in[k]);
         if (ioff[k] == SIZE_MAX) continue;
         din[k] = reinterpret_cast<const float *>(scratch.dev + ioff[k]);
-        e = cudaMemcpyAsync(scratch.dev + ioff[k], in[k], isz[k], cudaMemcpyHostToDevice, s);
+        e = cudaMemcpyAsync(scratch.dev + ioff[k], in[k], isz[k], cudaMemcpyDefault, s);
     }
     float *dout[3];
     for (int k = 0; k < 3; k++)
@@ -1966,8 +1979,15 @@ nbody_status nbody_mlp_eval(int64_t n, const float *features, const float *targe
                                   dout[0]);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "nbody_mlp_eval");
-    for (int k = 0; k < 3; k++)
-        if (ooff[k] != SIZE_MAX) std::memcpy(out[k], scratch.host + ooff[k], osz[k]);
+    for (int k = 0; k < 3; k++) {
+        if (ooff[k] == SIZE_MAX) continue;
+        if (is_device_ptr(out[k])) {  // another device's memory
+            e = cudaMemcpy(out[k], scratch.host + ooff[k], osz[k], cudaMemcpyDefault);
+            if (e != cudaSuccess) return cuda_fail(nullptr, e, "nbody_mlp_eval");
+        } else {
+            std::memcpy(out[k], scratch.host + ooff[k], osz[k]);
+        }
+    }
     return NBODY_OK;
 }
 
