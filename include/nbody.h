@@ -377,7 +377,11 @@ nbody_status nbody_mlp_predict(nbody_ctx *ctx, float *pred, float *features, int
  * [NBODY_MLP_PARAMS] (FP32, rounded to BF16 inside, as the training kernels
  * use them), norm [16] (feature means then standard deviations; NULL = none).
  * Outputs (host or device, nullable): pred [n], grad [NBODY_MLP_PARAMS] of the
- * mean loss, loss (one float).  Errors: EINVAL, ENOMEM, ECUDA. */
+ * mean loss, loss (one float).  Arrays of the current device are used in place;
+ * scratch comes from a stream-ordered pool (at most 32 MB kept per device) and
+ * page-locked blocks (at most four kept), both given back when a context is
+ * destroyed; calls may run on several threads and streams at once.
+ * Errors: EINVAL, ENOMEM, ECUDA. */
 nbody_status nbody_mlp_eval(int64_t n, const float *features, const float *targets,
                             const float *params, const float *norm, float *pred, float *grad,
                             float *loss, void *cuda_stream);
