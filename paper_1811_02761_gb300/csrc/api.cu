@@ -598,7 +598,7 @@ bool use_compensation(const nbody_config &c) {
 // Which walk: up to kCoopParticles particles only the cooperative kernel is
 // launched; above, the one-warp kernel, then the cooperative one for the
 // groups cut at the quota -- or for all of them when at most kCoopGroups are
-// walked (a block step's active groups; the kernels read the count).
+// walked (the kernels read the count).  Block steps: walk_ordered.cuh.
 // The line lies where the two meet: galaxy, walk only, one warp per group
 // against cooperative: N = 4096 0.198 / 0.041 ms, 30000 0.24 / 0.10, 65536
 // 0.28 / 0.15, 131072 (2953 groups) 0.28 / 0.23, 262147 (5850) 0.37 / 0.41,
@@ -654,7 +654,7 @@ cudaError_t ensure_coop(nbody_ctx *c) {
 }
 
 WalkShape walk_shape(nbody_ctx *c, bool geometric, bool phi, bool safe) {
-    WalkShape sh;
+    WalkShape sh{};
     sh.ipl = c->cfg.ipl;
     sh.geometric = geometric;
     sh.potential = phi;
@@ -805,11 +805,12 @@ nbody_status compute_order(nbody_ctx *c, const float *pcost, const int32_t **ord
 
 // Walk over the current groups; aold_s (sorted) must hold |a_old|, unless the
 // group pass has formed alpha and reset the queues already (prepared).
+// ordered (not with geometric or phi): the ordered walk.
 nbody_status run_walk(nbody_ctx *c, bool geometric, bool phi, bool safe, const int32_t *perm,
                       float *ax, float *ay, float *az, float *ph, float4 *acc_sorted,
                       bool reset_accumulators = true, const float *pcost = nullptr,
                       const int32_t *active_order = nullptr, const int32_t *nactive = nullptr,
-                      bool prepared = false) {
+                      bool prepared = false, bool ordered = false) {
     const int32_t *order = active_order;
     if (!geometric && !active_order) {
         nbody_status so = compute_order(c, pcost, &order);
@@ -829,7 +830,7 @@ nbody_status run_walk(nbody_ctx *c, bool geometric, bool phi, bool safe, const i
         NB_CUDA(c, cudaEventCreate(&ev));
         c->wev.push_back(ev);
     }
-    if (ensure_coop(c) != cudaSuccess) return fail(c, NBODY_ENOMEM, "allocation");
+    if (!ordered && ensure_coop(c) != cudaSuccess) return fail(c, NBODY_ENOMEM, "allocation");
     WalkArgs a = walk_args(c, geometric);
     a.order = order;
     a.nactive = nactive;
@@ -843,7 +844,9 @@ nbody_status run_walk(nbody_ctx *c, bool geometric, bool phi, bool safe, const i
     const bool gtime = c->capturing && c->gwev_used + 2 <= 4 && c->gwev[c->gwev_used];
     if (!c->capturing) NB_CUDA(c, cudaEventRecord(c->wev[c->wev_used], c->stream));
     if (gtime) NB_CUDA(c, cudaEventRecordWithFlags(c->gwev[c->gwev_used], c->stream, cudaEventRecordExternal));
-    cudaError_t e = launch_walk(c->stream, a, walk_shape(c, geometric, phi, safe), c->nsm);
+    WalkShape sh = walk_shape(c, geometric, phi, safe);
+    sh.ordered = ordered;
+    cudaError_t e = launch_walk(c->stream, a, sh, c->nsm);
     if (e != cudaSuccess) return cuda_fail(c, e, "walk launch");
     if (!c->capturing) {
         NB_CUDA(c, cudaEventRecord(c->wev[c->wev_used + 1], c->stream));
@@ -853,7 +856,7 @@ nbody_status run_walk(nbody_ctx *c, bool geometric, bool phi, bool safe, const i
         NB_CUDA(c, cudaEventRecordWithFlags(c->gwev[c->gwev_used + 1], c->stream, cudaEventRecordExternal));
         c->gwev_used += 2;
     }
-    c->kernels += (c->L.n <= kCoopParticles ? 1 : 2) + (c->L.n > kCutQuota ? 1 : 0);
+    c->kernels += ordered ? 1 : (c->L.n <= kCoopParticles ? 1 : 2) + (c->L.n > kCutQuota ? 1 : 0);
     if (!geometric) c->costs_valid = true;
     return NBODY_OK;
 }
@@ -1232,8 +1235,10 @@ static nbody_status block_steps(nbody_ctx *ctx, const Layout &L, StepState *S, i
         launch_block_active_groups(q, ctx->ds, P<int32_t>(ctx->grp_first), P<int32_t>(ctx->grp_count),
                                    S[cur].lvl, T, K, P<int32_t>(ctx->grp_order), dact, ctx->nsm);
         ctx->kernels += 1;
+        // particles on several levels: the ordered walk.  All on level 0: these
+        // are shared steps, and walked as those are
         st = run_walk(ctx, false, false, safe, nullptr, nullptr, nullptr, nullptr, nullptr, acc,
-                      false, nullptr, P<int32_t>(ctx->grp_order), dact, true);
+                      false, nullptr, P<int32_t>(ctx->grp_order), dact, true, kmax > 0);
         if (st != NBODY_OK) return st;
         NB_CUDA(ctx, pool_event(ctx, &e2));
         NB_CUDA(ctx, cudaEventRecord(e2, q));

@@ -335,6 +335,7 @@ struct WalkShape {
     bool quad;                  // accepted nodes add their quadrupole
     int warps_per_block;
     bool coop_only;             // host: the walk has few enough particles for the cooperative kernel alone
+    bool ordered;               // the ordered walk alone (no potential, |a_old| given)
     int *warps_launched;        // host, nullable: receives the resident walk warps
 };
 // The walk of one warp per group (not with sh.coop_only), then the

@@ -25,7 +25,16 @@ NB_COOP_EXTERN(1, true) NB_COOP_EXTERN(2, true) NB_COOP_EXTERN(3, true) NB_COOP_
 #undef NB_COOP_EXTERN
 
 template <int IPL, bool QUAD>
+cudaError_t launch_ordered_ipl(cudaStream_t s, const WalkArgs &a, const WalkShape &sh, int nsm);
+#define NB_ORDERED_EXTERN(I, Q) \
+    extern template cudaError_t launch_ordered_ipl<I, Q>(cudaStream_t, const WalkArgs &, const WalkShape &, int);
+NB_ORDERED_EXTERN(1, false) NB_ORDERED_EXTERN(2, false) NB_ORDERED_EXTERN(3, false) NB_ORDERED_EXTERN(4, false)
+NB_ORDERED_EXTERN(1, true) NB_ORDERED_EXTERN(2, true) NB_ORDERED_EXTERN(3, true) NB_ORDERED_EXTERN(4, true)
+#undef NB_ORDERED_EXTERN
+
+template <int IPL, bool QUAD>
 static cudaError_t launch_both(cudaStream_t s, const WalkArgs &a, const WalkShape &sh, int nsm) {
+    if (sh.ordered) return launch_ordered_ipl<IPL, QUAD>(s, a, sh, nsm);
     if (!sh.coop_only) {
         const cudaError_t e = launch_walk_ipl<IPL, QUAD>(s, a, sh, nsm);
         if (e != cudaSuccess) return e;

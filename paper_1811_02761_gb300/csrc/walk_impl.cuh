@@ -83,8 +83,9 @@ struct ISlots {
 // entries: the entry pairs k0, k0 + ks, k0 + 2 ks, ... (see the lane tiling
 // below).  Plain sums accumulate straight into the packed running sums; with
 // COMP each flush forms packed partial sums that are folded into the running
-// sums at its end with Neumaier compensation.
-template <int J0, int NQ, int IPL, bool PHI, bool COMP, bool SAFE>
+// sums at its end with Neumaier compensation.  ORD: the products in the order
+// of the ordered walk (walk_ordered.cuh).
+template <int J0, int NQ, int IPL, bool PHI, bool COMP, bool SAFE, bool ORD>
 __device__ __forceinline__ void flush_list(float4 *L, int nl, float eps2, int k0, int ks,
                                            ISlots<IPL> &I) {
     if (nl & 1) {  // pad to a whole pair with a massless, distant entry
@@ -132,7 +133,7 @@ __device__ __forceinline__ void flush_list(float4 *L, int nl, float eps2, int k0
             // 15.0 FP32 lane cycles per interaction; walk at N = 2^23 6.19 ->
             // 6.13 ms)
             const float2 mr = __fmul2_rn(pm, ri);
-            const float2 w3 = __fmul2_rn(mr, __fmul2_rn(ri, ri));
+            const float2 w3 = ORD ? __fmul2_rn(__fmul2_rn(mr, ri), ri) : __fmul2_rn(mr, __fmul2_rn(ri, ri));
             sx[q] = __ffma2_rn(w3, dx, sx[q]);
             sy[q] = __ffma2_rn(w3, dy, sy[q]);
             sz[q] = __ffma2_rn(w3, dz, sz[q]);
@@ -299,7 +300,7 @@ __device__ __forceinline__ Tiling lane_tiling(int cnt, int warp = 0) {
 // The flush loops of the runs from slot J on (run K).  KM: how many warps
 // share the list (the stride of a lane's entry pairs is KM times the run's
 // splits; t.k0 then counts the warp in).
-template <int J, int K, int IPL, bool PHI, bool COMP, bool SAFE, bool QUADL, int KM = 1>
+template <int J, int K, int IPL, bool PHI, bool COMP, bool SAFE, bool QUADL, int KM = 1, bool ORD = false>
 __device__ __forceinline__ void flush_runs(const Tiling &t, float4 *L, int nl, float eps2,
                                            ISlots<IPL> &I) {
     if constexpr (J < IPL && K < 3) {
@@ -308,19 +309,19 @@ __device__ __forceinline__ void flush_runs(const Tiling &t, float4 *L, int nl, f
 #define NB_FLUSH(R)                                                                            \
     do {                                                                                       \
         if constexpr (QUADL) flush_quad_list<J, R, IPL, PHI, COMP, SAFE>(L, nl, eps2, k0, ks, I); \
-        else flush_list<J, R, IPL, PHI, COMP, SAFE>(L, nl, eps2, k0, ks, I);                  \
+        else flush_list<J, R, IPL, PHI, COMP, SAFE, ORD>(L, nl, eps2, k0, ks, I);             \
     } while (0)
         if constexpr (J + 4 <= IPL) {
             if (r == 4) { NB_FLUSH(4); return; }
         }
         if constexpr (J + 3 <= IPL) {
-            if (r == 3) { NB_FLUSH(3); flush_runs<J + 3, K + 1, IPL, PHI, COMP, SAFE, QUADL, KM>(t, L, nl, eps2, I); return; }
+            if (r == 3) { NB_FLUSH(3); flush_runs<J + 3, K + 1, IPL, PHI, COMP, SAFE, QUADL, KM, ORD>(t, L, nl, eps2, I); return; }
         }
         if constexpr (J + 2 <= IPL) {
-            if (r == 2) { NB_FLUSH(2); flush_runs<J + 2, K + 1, IPL, PHI, COMP, SAFE, QUADL, KM>(t, L, nl, eps2, I); return; }
+            if (r == 2) { NB_FLUSH(2); flush_runs<J + 2, K + 1, IPL, PHI, COMP, SAFE, QUADL, KM, ORD>(t, L, nl, eps2, I); return; }
         }
         NB_FLUSH(1);
-        flush_runs<J + 1, K + 1, IPL, PHI, COMP, SAFE, QUADL, KM>(t, L, nl, eps2, I);
+        flush_runs<J + 1, K + 1, IPL, PHI, COMP, SAFE, QUADL, KM, ORD>(t, L, nl, eps2, I);
 #undef NB_FLUSH
     }
 }

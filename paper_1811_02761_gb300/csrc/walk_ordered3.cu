@@ -1,0 +1,8 @@
+// walk_ordered3.cu -- instances of the ordered walk with up to 3 i-particles per
+// lane, monopole nodes (separate translation unit so the instances compile
+// in parallel).
+#include "walk_ordered.cuh"
+
+namespace nb {
+template cudaError_t launch_ordered_ipl<3, false>(cudaStream_t, const WalkArgs &, const WalkShape &, int);
+}  // namespace nb

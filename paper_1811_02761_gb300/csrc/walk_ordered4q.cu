@@ -1,0 +1,8 @@
+// walk_ordered4q.cu -- instances of the ordered walk with up to 4 i-particles per
+// lane, nodes with quadrupoles (separate translation unit so the instances compile
+// in parallel).
+#include "walk_ordered.cuh"
+
+namespace nb {
+template cudaError_t launch_ordered_ipl<4, true>(cudaStream_t, const WalkArgs &, const WalkShape &, int);
+}  // namespace nb
