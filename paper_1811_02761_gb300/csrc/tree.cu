@@ -486,7 +486,8 @@ __device__ __forceinline__ bool internal_nodes(const Layout &L, bool go, int p, 
 
 // Count a finished node in at its parent `par`; the caller has fenced the
 // node's records before, and the lane that completes the parent fences after
-// it, so it sees every child's records.  (A relaxed add between the two fences:
+// it and passes a warp barrier, so the lanes of its warp see every child's
+// records.  (A relaxed add between the two fences:
 // an add with release and acquire semantics would fence a second time on every
 // level of the climb.)  Returns how many of the parent's children have arrived.
 __device__ __forceinline__ int count_in(int par, int32_t *node_arrive) {
@@ -625,9 +626,10 @@ __global__ void __launch_bounds__(256, NB_MOMENTS_MIN_CTAS) moments_kernel(
             }
         }
         // internal nodes: the chunk's leaf records are device-visible before
-        // any lane counts a leaf in (the warp barrier, then the lane's fence).  A climbing thread carries a member key (its leaf's first
-        // particle): every ancestor's cell follows from it and the ancestor's
-        // level, one up per step.
+        // any lane counts a leaf in (the warp barrier, then the lane's fence).
+        // A climbing thread carries a member key (its leaf's first particle):
+        // every ancestor's cell follows from it and the ancestor's level, one
+        // up per step.
         __syncwarp();
         __threadfence();
         int node = id0, par = -1, level = 0;
@@ -652,7 +654,11 @@ __global__ void __launch_bounds__(256, NB_MOMENTS_MIN_CTAS) moments_kernel(
                     ready = count_in(par, node_arrive) == nc;
                 }
             }
+            // the completing lane's fence, then a warp barrier (ballots and
+            // shuffles order no memory): the team's lanes, which read the
+            // children, come after every child's count-in
             if (ready) __threadfence();
+            __syncwarp();
             unsigned rm = __ballot_sync(NB_FULL, ready);
             if (!rm) break;
             while (rm) {  // four parents at a time, eight lanes each
