@@ -140,12 +140,16 @@ __global__ void __launch_bounds__(256) bbox_kernel(int64_t n, const T *__restric
     }
     if (!done) return;
     __shared__ int last;
-    __threadfence();  // this thread's extents before the block counts itself in
+    // the fences are the counting thread's, inside the barriers: they cover the
+    // whole block's extents before and its reads after
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(done, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
     __syncthreads();
     if (!last) return;
-    __threadfence();
     for (int s = threadIdx.x; s < nsys; s += blockDim.x) bbox_finalize(s, levels, boxord, box);
     if (threadIdx.x == 0) *done = 0;
 }
@@ -163,7 +167,6 @@ __global__ void __launch_bounds__(BX_T) bbox_one_kernel(int64_t n, const T *__re
                                                         const T *__restrict__ z, uint32_t *boxord,
                                                         int levels, SysBox *box, uint32_t *done) {
     __shared__ uint32_t sh[6][BX_T / 32];
-    __shared__ int last;
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     const int64_t step = (int64_t)gridDim.x * (BX_T * BX_IPT);
     for (int64_t base = (int64_t)blockIdx.x * (BX_T * BX_IPT) + threadIdx.x; base < n; base += step) {
@@ -201,13 +204,12 @@ __global__ void __launch_bounds__(BX_T) bbox_one_kernel(int64_t n, const T *__re
             r = threadIdx.x < 3 ? min(r, sh[threadIdx.x][k]) : max(r, sh[threadIdx.x][k]);
         if (threadIdx.x < 3) atomicMin(&boxord[threadIdx.x], r);
         else atomicMax(&boxord[threadIdx.x], r);
-        __threadfence();
     }
     if (w != 0) return;
     __syncwarp();
-    if (lane == 0) last = atomicAdd(done, 1u) == gridDim.x - 1;
-    __syncwarp();
-    if (!last || lane != 0) return;
+    if (lane != 0) return;
+    __threadfence();  // after the warp barrier: covers the extents of all six lanes
+    if (atomicAdd(done, 1u) != gridDim.x - 1) return;
     __threadfence();
     bbox_finalize(0, levels, boxord, box);
     *done = 0;

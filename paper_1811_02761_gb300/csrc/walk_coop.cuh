@@ -338,13 +338,16 @@ __global__ void __maxnreg__((walk_regs<IPL, QUAD || COMP>()))
                 __stcg(&a.part[(size_t)task * kPartStride + i], make_float4(r[0], r[1], r[2], r[3]));
             }
             if (tid == 0) a.part_entries[task] = (int32_t)total;
-            __threadfence();
+            // the fences are the counting thread's, inside the barriers: they
+            // cover the writes of the whole CTA before and its reads after
             __syncthreads();
-            if (tid == 0)
+            if (tid == 0) {
+                __threadfence();
                 s_last = atomicAdd(&a.part_arrive[owner], 1) == P * (second ? a.cut_count[owner] : 1) - 1;
+                __threadfence();
+            }
             __syncthreads();
             finish = s_last != 0;
-            if (finish) __threadfence();
         }
         if (finish) {
             // parts of the group: slots rec_i P + k; in the second stage those
