@@ -548,7 +548,8 @@ __global__ void __launch_bounds__(32 * RK_WARPS) rank_sort_kernel(const uint64_t
 
 cudaError_t rank_sort(cudaStream_t s, const uint64_t *keys, int64_t n, uint64_t *kout, uint32_t *vout) {
     const size_t smem = (size_t)n * 8;
-    if (smem > 48 * 1024) {
+    // 48 KB, the kernel's static 1 KB included, need no asking
+    if (smem > 47 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(rank_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    kRankSortMax * 8);
         if (e != cudaSuccess) return e;

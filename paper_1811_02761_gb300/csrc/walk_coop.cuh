@@ -424,7 +424,8 @@ cudaError_t launch_coop_ipl(cudaStream_t s, const WalkArgs &a, const WalkShape &
         else k = sh.safe ? coop_walk_kernel<IPL, false, false, true, QUAD> : coop_walk_kernel<IPL, false, false, false, QUAD>;
     }
     cudaError_t err = cudaSuccess;
-    if (smem > 48 * 1024) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the kernel's static words count towards the 48 KB that need no asking)
+    if (smem > 47 * 1024) err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     // resident CTAs, from the register and shared-memory budgets (no CTA waits
     // for another, so a grid larger than that would only queue); an occupancy
