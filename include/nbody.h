@@ -377,7 +377,8 @@ nbody_status nbody_mlp_predict(nbody_ctx *ctx, float *pred, float *features, int
  * [NBODY_MLP_PARAMS] (FP32, rounded to BF16 inside, as the training kernels
  * use them), norm [16] (feature means then standard deviations; NULL = none).
  * Outputs (host or device, nullable): pred [n], grad [NBODY_MLP_PARAMS] of the
- * mean loss, loss (one float).  Arrays of the current device are used in place;
+ * mean loss, loss (one float).  Arrays of the current device are used in place,
+ * except inputs that an output overlaps and outputs that overlap each other;
  * scratch comes from a stream-ordered pool (at most 32 MB kept per device) and
  * page-locked blocks (at most four kept), both given back when a context is
  * destroyed; calls may run on several threads and streams at once.

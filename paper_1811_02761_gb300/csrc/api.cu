@@ -1943,23 +1943,33 @@ nbody_status nbody_mlp_eval(int64_t n, const float *features, const float *targe
     // behind the partial sums; host outputs are written by the kernels into
     // page-locked memory and copied from there (three copies into pageable
     // memory took 100 us at n = 60013, allocating and freeing the device block
-    // another 100).
+    // another 100).  Arrays may share memory: an input that an output overlaps
+    // is staged too, and so is an output that overlaps another (the loss, then
+    // the gradient, is the one that stays).
     auto align = [](size_t v) { return (v + 255) & ~(size_t)255; };
+    auto overlap = [](const void *p, size_t pb, const void *q, size_t qb) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(q);
+        return p && q && a < b + qb && b < a + pb;
+    };
     size_t dev = align((size_t)nb * psz) + align((size_t)nb * 4), host = 0;
     int dev_id = 0;
     if (cudaGetDevice(&dev_id) != cudaSuccess) return fail(nullptr, NBODY_ECUDA, "no device");
     const void *in[4] = {features, targets, params, norm};
     const size_t isz[4] = {fsz, tsz, psz, 64};
     size_t ioff[4];
-    for (int k = 0; k < 4; k++) {
-        ioff[k] = in[k] && !on_device(in[k], dev_id) ? dev : SIZE_MAX;
-        if (ioff[k] != SIZE_MAX) dev += align(isz[k]);
-    }
     void *out[3] = {pred, grad, loss};
     const size_t osz[3] = {tsz, psz, 4};
     size_t ooff[3];
+    for (int k = 0; k < 4; k++) {
+        bool stage = !on_device(in[k], dev_id);
+        for (int j = 0; j < 3; j++) stage = stage || overlap(in[k], isz[k], out[j], osz[j]);
+        ioff[k] = in[k] && stage ? dev : SIZE_MAX;
+        if (ioff[k] != SIZE_MAX) dev += align(isz[k]);
+    }
     for (int k = 0; k < 3; k++) {
-        ooff[k] = out[k] && !on_device(out[k], dev_id) ? host : SIZE_MAX;
+        bool stage = !on_device(out[k], dev_id);
+        for (int j = 0; j < 3; j++) stage = stage || (j != k && overlap(out[k], osz[k], out[j], osz[j]));
+        ooff[k] = out[k] && stage ? host : SIZE_MAX;
         if (ooff[k] != SIZE_MAX) host += align(osz[k]);
     }
     nb::Scratch scratch(s);
@@ -1986,7 +1996,7 @@ nbody_status nbody_mlp_eval(int64_t n, const float *features, const float *targe
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "nbody_mlp_eval");
     for (int k = 0; k < 3; k++) {
         if (ooff[k] == SIZE_MAX) continue;
-        if (is_device_ptr(out[k])) {  // another device's memory
+        if (is_device_ptr(out[k])) {  // another device's memory, or shared by two outputs
             e = cudaMemcpy(out[k], scratch.host + ooff[k], osz[k], cudaMemcpyDefault);
             if (e != cudaSuccess) return cuda_fail(nullptr, e, "nbody_mlp_eval");
         } else {
