@@ -1992,7 +1992,7 @@ nbody_status nbody_mlp_eval(int64_t n, const float *features, const float *targe
         e = launch_mlp_train_step(s, din[0], din[1], 0, 1, (int)n, nullptr, din[2], din[3], gpart, lpart,
                                   dout[1], dout[2], nullptr, nullptr, nullptr, nullptr, 0.0f, 1, false,
                                   dout[0]);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = scratch.finish();
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "nbody_mlp_eval");
     for (int k = 0; k < 3; k++) {
         if (ooff[k] == SIZE_MAX) continue;

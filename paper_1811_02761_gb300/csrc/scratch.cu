@@ -80,7 +80,13 @@ cudaError_t Scratch::take(size_t dev_bytes, size_t host_bytes) {
     return cudaSuccess;
 }
 
+cudaError_t Scratch::finish() {
+    finished_ = true;
+    return cudaStreamSynchronize(stream_);
+}
+
 Scratch::~Scratch() {
+    if (!finished_) cudaStreamSynchronize(stream_);
     if (dev) cudaFreeAsync(dev, stream_);
     if (!host) return;
     {
