@@ -4,7 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <climits>
+#include <cstdint>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -40,6 +40,8 @@ struct GraphKey {
     float dt;
     bool safe;
     bool mlp_norm;  // the cost model's input statistics were set at capture
+    bool coop;      // the walk captured, and whether groups may be cut: they
+    int64_t sys_max;  // depend on the sizes of the systems
     nbody_config cfg;
     int64_t growths;  // buffers may move, and only some of them, when one grows
     const void *bufs[9];
@@ -95,6 +97,8 @@ struct nbody_ctx {
     double *h_diag = nullptr;  // pinned
     char *h_sys = nullptr;     // pinned: offsets, eps, eps^2 on their way to the device
     size_t h_sys_bytes = 0;
+    int64_t sys_max = 0;   // particles of the largest system of the last build or step
+    double sys_mean = 0;   // and of the system that a particle is in, on average
     cudaEvent_t sys_ev = nullptr;
 
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -499,10 +503,15 @@ nbody_status upload_systems(nbody_ctx *c, int nsys, const int64_t *offsets, cons
     int64_t *off = reinterpret_cast<int64_t *>(c->h_sys);
     float *e1 = reinterpret_cast<float *>(c->h_sys + ob), *e2 = e1 + nsys;
     std::memcpy(off, offsets, ob);
+    c->sys_max = 0;
+    c->sys_mean = 0.0;
     for (int s = 0; s < nsys; s++) {
         const float e = eps_sys ? eps_sys[s] : c->cfg.eps;
         e1[s] = e;
         e2[s] = e * e;
+        const int64_t ns = offsets[s + 1] - offsets[s];
+        c->sys_max = std::max(c->sys_max, ns);
+        c->sys_mean += (double)ns * (double)ns / (double)std::max<int64_t>(offsets[nsys], 1);
     }
     NB_CUDA(c, cudaMemcpyAsync(c->sys_off.p, off, ob, cudaMemcpyHostToDevice, c->stream));
     NB_CUDA(c, cudaMemcpyAsync(c->sys_eps2.p, e2, eb, cudaMemcpyHostToDevice, c->stream));
@@ -595,17 +604,37 @@ bool use_compensation(const nbody_config &c) {
     return c.compensated == 1 || (c.compensated == 2 && c.delta_acc <= kAutoCompensateDacc);
 }
 
-// Which walk: up to kCoopParticles particles only the cooperative kernel is
-// launched; above, the one-warp kernel, then the cooperative one for the
-// groups cut at the quota -- or for all of them when at most kCoopGroups are
-// walked (the kernels read the count).  Block steps: walk_ordered.cuh.
-// The line lies where the two meet: galaxy, walk only, one warp per group
-// against cooperative: N = 4096 0.198 / 0.041 ms, 30000 0.24 / 0.10, 65536
-// 0.28 / 0.15, 131072 (2953 groups) 0.28 / 0.23, 262147 (5850) 0.37 / 0.41,
-// 1000003 0.98 / 1.38: once every warp has a group of its own, the barriers
-// of the cooperative walk only cost.
-constexpr int64_t kCoopParticles = 1 << 17;
-constexpr int kCoopGroups = 3000;
+// Entries of an ordinary group's list: 1500 at delta_acc = 2^-9, growing with
+// delta_acc^-0.485 (measured from 2^-1 to 2^-20), and with theta^-3 for the
+// geometric criterion.
+double ordinary_list(const nbody_ctx *c, bool geometric) {
+    return 1500.0 * (geometric ? std::pow(0.5 / c->cfg.theta, 3.0)
+                               : std::pow(std::max(c->cfg.delta_acc, 1e-12f) * 512.0, -0.485));
+}
+
+// Which walk: the cooperative one for all groups, or one warp per group with
+// the cooperative one for the groups cut at the quota.  (Block steps:
+// walk_ordered.cuh.)  One warp per group takes as long as the longest list's
+// chain, a launch and 0.05 + 0.0014 G us per entry, as long as most warps have
+// one group; the cooperative walk a launch (more with quadrupoles or
+// compensated sums) and a time per group that grows with its list.  Lists are
+// estimated by ordinary_list and the particles of a system, the groups as
+// 0.7 G particles each and at least one per system.  Fitted to 1040 walks of
+// 2 to 200003 particles, 1 to 16000 systems, groups of 16 to 96, quadrupoles,
+// compensated sums and delta_acc = 2^-14 to 2^-5: within 3 % of the better one
+// of the two (geometric mean; a line by particles alone, 2^17, was 28 %
+// off).  Both sides in us, one warp / cooperative: galaxy, G = 64, N = 4096
+// 187 / 41, 100003 252 / 201, 200003 318 / 350; N = 100003, G = 16 146 / 396; 12000
+// systems of 10 particles 34 / 181; 256 particles, compensated, 25 / 42.
+bool coop_walk(const nbody_ctx *c, bool geometric) {
+    const double G = c->cfg.group_size, ordinary = ordinary_list(c, geometric);
+    const double groups = c->L.n / (0.7 * G) + c->L.nsys;
+    const bool more = c->cfg.quadrupole != 0 || use_compensation(c->cfg);
+    const double chain = 5.0 + std::min((double)c->sys_max, ordinary) * (0.05 + 0.0014 * G);
+    const double coop = (more ? 70.0 : 30.0) +
+                        groups * (0.002 + std::min(c->sys_mean, ordinary) * (2.5e-5 + 2e-7 * G));
+    return coop < chain;
+}
 
 // Records for groups cut at the quota: twice the count of groups of G
 // particles (they hold 0.7 G on average), so a walk of more groups, which is
@@ -616,15 +645,12 @@ int64_t heavy_records(const nbody_ctx *c) { return 2 * c->L.n / c->cfg.group_siz
 // cooperative kernel.  A group is one warp's serial chain (40-80 ns per
 // entry), so one far longer than the others runs alone at the end of the
 // launch (Plummer, N = 262147, no |a_old|: one group of 167,663 entries took
-// 13 of the walk's 14 ms).  The line is 2.7 ordinary lists (1500 entries at
-// delta_acc = 2^-9, growing with delta_acc^-0.485, measured from 2^-1 to
-// 2^-20, and with theta^-3 for the geometric criterion), below which the tail
+// 13 of the walk's 14 ms).  The line is 2.7 ordinary lists, below which the tail
 // is an ordinary group's.  With n / G groups on a few thousand warps a tail
 // of 0.38 n / G entries (half of what a warp walks in all) is the line: a forest
 // of 512 systems walks in 9.35 ms (10.0 at 0.5 n / G, 11.6 uncut).
 int list_quota(const nbody_ctx *c, bool geometric) {
-    const double q = geometric ? std::pow(0.5 / c->cfg.theta, 3.0)
-                               : std::pow(std::max(c->cfg.delta_acc, 1e-12f) * 512.0, -0.485);
+    const double q = ordinary_list(c, geometric) / 1500.0;
     return (int)std::min(std::max(4096.0 * std::max(q, 1.0), 0.38 * c->L.n / c->cfg.group_size), 1e9);
 }
 
@@ -633,8 +659,14 @@ int list_quota(const nbody_ctx *c, bool geometric) {
 // 1.01 ms at 2048 and 4096, 1.06 at 8192, 1.10 at 16384).
 constexpr int kCutQuota = 4096;
 
-cudaError_t ensure_coop(nbody_ctx *c) {
+// A list holds every particle of its system at most once: no group is cut
+// where the largest system is within the quota.
+bool cuts_groups(const nbody_ctx *c, bool geometric) { return c->sys_max > list_quota(c, geometric); }
+
+cudaError_t ensure_coop(nbody_ctx *c, bool geometric) {
     cudaError_t e = cudaSuccess;
+    const bool coop = coop_walk(c, geometric);
+    if (!coop && !cuts_groups(c, geometric)) return e;
     if (!c->part_ctl.p) {
         e = ensure(c->part, (size_t)kCutTasks * kPartStride * sizeof(float4));
         if (e == cudaSuccess) e = ensure(c->cut, (size_t)kCutTasks * kCutWords * 4);
@@ -645,7 +677,7 @@ cudaError_t ensure_coop(nbody_ctx *c) {
         if (e == cudaSuccess)
             e = cudaMemsetAsync(P<int32_t>(c->part_ctl) + kCutTasks, 0, (size_t)kCutTasks * 2 * 4, c->stream);
     }
-    if (e == cudaSuccess && c->L.n > kCoopParticles) {
+    if (e == cudaSuccess && !coop) {
         const size_t bytes = (size_t)heavy_records(c) * kHeavyWords * 4;
         if (c->heavy.bytes < bytes) c->growths++;
         e = ensure(c->heavy, bytes);
@@ -661,7 +693,7 @@ WalkShape walk_shape(nbody_ctx *c, bool geometric, bool phi, bool safe) {
     sh.compensated = use_compensation(c->cfg);
     sh.safe = safe;
     sh.quad = c->cfg.quadrupole != 0;
-    sh.coop_only = c->L.n <= kCoopParticles;
+    sh.coop_only = coop_walk(c, geometric);
     sh.warps_per_block = c->cfg.warps_per_block;
     sh.warps_launched = &c->walk_warps;
     return sh;
@@ -689,11 +721,12 @@ WalkArgs walk_args(nbody_ctx *c, bool geometric) {
     a.theta = c->cfg.theta;
     a.list_depth = c->cfg.list_depth;
     a.stack_depth = c->cfg.stack_depth;
-    a.coop_groups = c->L.n <= kCoopParticles ? INT32_MAX : kCoopGroups;
+    a.coop_all = coop_walk(c, geometric);
+    a.longest = c->sys_max;
     a.heavy = P<uint32_t>(c->heavy);  // only the one-warp kernel cuts groups into it
     a.quota = list_quota(c, geometric);
     a.cut_quota = kCutQuota;
-    a.heavy_cap = (int)std::min<int64_t>(heavy_records(c), INT32_MAX);
+    a.heavy_cap = a.longest > a.quota ? (int)std::min<int64_t>(heavy_records(c), INT32_MAX) : 0;
     a.coop_target[0] = std::min(c->nsm * kCoopTarget, kCutTasks);
     a.coop_target[1] = std::min(c->nsm * kCoopTarget2, kCutTasks);
     a.cut = P<uint32_t>(c->cut);
@@ -830,7 +863,7 @@ nbody_status run_walk(nbody_ctx *c, bool geometric, bool phi, bool safe, const i
         NB_CUDA(c, cudaEventCreate(&ev));
         c->wev.push_back(ev);
     }
-    if (!ordered && ensure_coop(c) != cudaSuccess) return fail(c, NBODY_ENOMEM, "allocation");
+    if (!ordered && ensure_coop(c, geometric) != cudaSuccess) return fail(c, NBODY_ENOMEM, "allocation");
     WalkArgs a = walk_args(c, geometric);
     a.order = order;
     a.nactive = nactive;
@@ -856,7 +889,7 @@ nbody_status run_walk(nbody_ctx *c, bool geometric, bool phi, bool safe, const i
         NB_CUDA(c, cudaEventRecordWithFlags(c->gwev[c->gwev_used + 1], c->stream, cudaEventRecordExternal));
         c->gwev_used += 2;
     }
-    c->kernels += ordered ? 1 : (c->L.n <= kCoopParticles ? 1 : 2) + (c->L.n > kCutQuota ? 1 : 0);
+    c->kernels += ordered ? 1 : a.coop_all ? (a.longest > kCutQuota ? 2 : 1) : (a.longest > a.quota ? 3 : 1);
     if (!geometric) c->costs_valid = true;
     return NBODY_OK;
 }
@@ -1438,6 +1471,8 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
         key.dt = dt;
         key.safe = safe;
         key.mlp_norm = ctx->mlp_norm_set;
+        key.coop = coop_walk(ctx, false);
+        key.sys_max = ctx->sys_max;
         key.cfg = ctx->cfg;
         key.bufs[0] = ctx->keys.p;
         key.bufs[1] = ctx->vals.p;

@@ -313,7 +313,8 @@ struct WalkArgs {
     float *ax, *ay, *az, *phi;
     float4 *acc_sorted;        // (ax, ay, az, phi)
     // cooperative walk
-    int coop_groups;           // at most this many groups: all of them cooperatively
+    bool coop_all;             // every group cooperatively, not those cut at the quota
+    int64_t longest;           // no list has more entries
     uint32_t *heavy;           // records of the groups cut at the quota
     int quota, cut_quota;      // list entries after which a group, a part of a group is cut
     int heavy_cap;             // records (no quota for a walk of more groups)
@@ -334,7 +335,7 @@ struct WalkShape {
     bool safe;                  // some eps == 0: guard the self term
     bool quad;                  // accepted nodes add their quadrupole
     int warps_per_block;
-    bool coop_only;             // host: the walk has few enough particles for the cooperative kernel alone
+    bool coop_only;             // the cooperative kernel alone (WalkArgs::coop_all)
     bool ordered;               // the ordered walk alone (no potential, |a_old| given)
     int *warps_launched;        // host, nullable: receives the resident walk warps
 };

@@ -37,7 +37,7 @@ static cudaError_t launch_both(cudaStream_t s, const WalkArgs &a, const WalkShap
     if (sh.ordered) return launch_ordered_ipl<IPL, QUAD>(s, a, sh, nsm);
     if (!sh.coop_only) {
         const cudaError_t e = launch_walk_ipl<IPL, QUAD>(s, a, sh, nsm);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || a.longest <= a.quota) return e;  // nothing can be cut
     }
     return launch_coop_ipl<IPL, QUAD>(s, a, sh, nsm);
 }

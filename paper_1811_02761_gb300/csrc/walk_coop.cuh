@@ -17,7 +17,8 @@
 //     particles (a few rounds, whose list entries only part 0 keeps) and
 //     walks every P-th of the child ranges found; the CTA that finishes last
 //     adds the P partial sums in part order.
-// It runs in two stages.  The first takes every group (few of them), or the
+// It runs in two stages.  The first takes every group (where coop_walk, api.cu,
+// says so), or the
 // groups the one-warp walk cut at its quota; a part whose own list passes
 // a.cut_quota entries is cut again, its open ranges recorded.  The second stage
 // walks those records, again with P CTAs each, to the end: however uneven the
@@ -81,7 +82,7 @@ __global__ void __maxnreg__((walk_regs<IPL, QUAD || COMP>()))
     int max_sp = 0;
     unsigned long long cta_entries = 0, cta_inter = 0, cta_quad = 0;
 
-    const bool all = !second && ng <= a.coop_groups;
+    const bool all = !second && a.coop_all;
     const int T = second ? ds->queue.ncut : (all ? ng : min(ds->queue.nheavy, a.heavy_cap));
     const int P = T > 0 ? max(1, min(kCoopParts, a.coop_target[second] / T)) : 1;
     const bool may_cut = !second && T <= kCutTasks / P;
@@ -440,7 +441,7 @@ cudaError_t launch_coop_ipl(cudaStream_t s, const WalkArgs &a, const WalkShape &
     if (sh.warps_launched && sh.coop_only) *sh.warps_launched = nsm * per_sm * kCoopWarps;
     k<<<nsm * per_sm, 32 * kCoopWarps, smem, s>>>(a, sh.geometric ? 1 : 0, 0);
     // a list no longer than the quota is never cut
-    if (a.n > a.cut_quota) k<<<nsm * per_sm, 32 * kCoopWarps, smem, s>>>(a, sh.geometric ? 1 : 0, 1);
+    if (a.longest > a.cut_quota) k<<<nsm * per_sm, 32 * kCoopWarps, smem, s>>>(a, sh.geometric ? 1 : 0, 1);
     return cudaGetLastError();
 }
 

@@ -507,7 +507,6 @@ __global__ void __maxnreg__((walk_regs<IPL, QUAD || COMP>())) walk_kernel(WalkAr
     const int ng = a.nactive ? *a.nactive : ds->ngroups;
     const int nnodes = ds->nnodes;
     const int npart = (int)a.n;
-    if (ng <= a.coop_groups) return;  // fewer groups than warps: the cooperative kernel's
     const unsigned lt = lanemask_lt();
     int max_sp = 0;
     unsigned long long warp_entries = 0, warp_inter = 0, warp_quad = 0;
