@@ -372,6 +372,18 @@ __device__ __forceinline__ void write_quad(int id, const float q[6], float4 *nod
 // from zero too; a node that fails its bounds check is still counted in at
 // its parent, which keeps every counter consistent.
 
+// Size b of an internal node at com from the child recurrence rec: bounded by
+// its widened cell unless the members may have left it (a refit).
+__device__ __forceinline__ float internal_size(const float (&com)[3], const CellF &cell, float rec, int refit) {
+    float c2 = 0.0f;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const float e = fabsf(com[a] - cell.c[a]) + cell.h;
+        c2 = fmaf(e, e, c2);
+    }
+    return (refit ? rec : fminf(rec, __fsqrt_ru(c2))) * kUp;
+}
+
 // One internal node per team of eight lanes from its children's records
 // (contiguous, at most 8), a lane per child; every lane of the warp calls this
 // (go false: a team without a node).  Sums run over the children in octant
@@ -382,10 +394,13 @@ __device__ __forceinline__ void write_quad(int id, const float q[6], float4 *nod
 // have left the cell) only the child recurrence bounds b.  Children finished
 // by other SMs in this launch are read past L1 (ld.global.cg): a sibling's
 // cache line may already sit in this SM's L1 from before it was written.
-// Bound by latency, as a climb is a chain of these: one thread per node, with
-// its 32 loads, eight square roots and eight-term double-float chain one after
-// the other, made the whole pass 35 us at n = 4096 and 47 us at 100003 (ncu);
-// with eight lanes it is 30 and 39 us.
+// Bound by latency, as a climb is a chain of these: one thread per node has 32
+// loads, eight square roots and an eight-term double-float chain one after the
+// other.  A node of few children is quicker by one lane (internal_node_alone).
+// Refit calls in us, one thread per node / eight lanes / eight lanes from four
+// children on: Plummer, N = 10^5 83 / 70 / 68, with quadrupoles 108 / 81 / 80;
+// 10^5 particles on 1000 points (chains of single children) 130 / 219 / 117; on a
+// line (one or two children) 279 / 292 / 204.
 // Records of a small tree's nodes in shared memory (moments_one_kernel).
 struct NodeRec {
     float4 A;
@@ -469,13 +484,7 @@ __device__ __forceinline__ bool internal_nodes(const Layout &L, bool go, int p, 
         }
     }
     if (ok && sub == 0) {
-        float c2 = 0.0f;
-#pragma unroll
-        for (int a = 0; a < 3; a++) {
-            const float e = fabsf(cp[a] - cell.c[a]) + cell.h;
-            c2 = fmaf(e, e, c2);
-        }
-        const float bp = (refit ? rec : fminf(rec, __fsqrt_ru(c2))) * kUp;
+        const float bp = internal_size(cp, cell, rec, refit);
         node_count[p] = count;
         write_node(p, cp[0], cp[1], cp[2], M, bp, G, c0, nc << 1, nodeA, nodeB, mass2);
         if (rec_s) rec_s[p] = NodeRec{make_float4(cp[0], cp[1], cp[2], M.x), M, count, bp};
@@ -484,15 +493,71 @@ __device__ __forceinline__ bool internal_nodes(const Layout &L, bool go, int p, 
     return ok || !go;
 }
 
-// Count a finished node in at its parent `par`; the caller has fenced the
-// node's records before, and the lane that completes the parent fences after
-// it and passes a warp barrier, so the lanes of its warp see every child's
-// records.  (A relaxed add between the two fences:
-// an add with release and acquire semantics would fence a second time on every
-// level of the climb.)  Returns how many of the parent's children have arrived.
+// The same for a node of at most kAlone children by one lane: same operations,
+// same order.
+constexpr int kAlone = 3;
+__device__ __forceinline__ bool internal_node_alone(const Layout &L, int p, int c0, int nc, int level,
+                                                    uint64_t key, int refit, int nn,
+                                                    const SysBox *__restrict__ box, float G,
+                                                    int32_t *node_count, float4 *nodeA, float4 *nodeB,
+                                                    float2 *mass2, float4 *nodeQ) {
+    if (c0 <= p || nc < 1 || nc > kAlone || c0 + nc > nn) return false;
+    const CellF cell = node_cell(L, key, level, box);
+    float4 A[kAlone];
+    float B[kAlone];
+    float2 M = make_float2(0.0f, 0.0f);
+    float px = 0.0f, py = 0.0f, pz = 0.0f;
+    int count = 0;
+#pragma unroll
+    for (int k = 0; k < kAlone; k++) {  // every field of every child in one round trip
+        const int j = k < nc ? c0 + k : c0;
+        A[k] = __ldcg(nodeA + j);
+        B[k] = __ldcg(&nodeB[j].x);
+        const float2 mk = __ldcg(mass2 + j);
+        const int ck = __ldcg(node_count + j);
+        if (k < nc) {
+            M = df_add(M, mk);
+            count += ck;
+            px = fmaf(A[k].w, A[k].x - cell.c[0], px);
+            py = fmaf(A[k].w, A[k].y - cell.c[1], py);
+            pz = fmaf(A[k].w, A[k].z - cell.c[2], pz);
+        }
+    }
+    float cp[3] = {cell.c[0], cell.c[1], cell.c[2]};
+    if (M.x > 0.0f) {
+        const float inv = 1.0f / M.x;
+        cp[0] = fmaf(px, inv, cp[0]); cp[1] = fmaf(py, inv, cp[1]); cp[2] = fmaf(pz, inv, cp[2]);
+    }
+    float rec = 0.0f;
+    float q[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < kAlone; k++) {
+        if (k < nc) {
+            const float dx = A[k].x - cp[0], dy = A[k].y - cp[1], dz = A[k].z - cp[2];
+            const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+            rec = fmaxf(rec, __fadd_ru(__fsqrt_ru(r2), B[k]));
+            if (nodeQ) {
+                const float4 q0 = __ldcg(nodeQ + 2 * (c0 + k)), q1 = __ldcg(nodeQ + 2 * (c0 + k) + 1);
+                q[0] += q0.x; q[1] += q0.y; q[2] += q0.z; q[3] += q0.w; q[4] += q1.x; q[5] += q1.y;
+                quad_add(q, A[k].w, dx, dy, dz, r2);
+            }
+        }
+    }
+    const float bp = internal_size(cp, cell, rec, refit);
+    node_count[p] = count;
+    write_node(p, cp[0], cp[1], cp[2], M, bp, G, c0, nc << 1, nodeA, nodeB, mass2);
+    if (nodeQ) write_quad(p, q, nodeQ);
+    return true;
+}
+
+// Count a finished node in at its parent `par`, with release and acquire
+// semantics: the node's records, and what other lanes wrote before a warp
+// barrier that this lane has passed, are published by it; and the lane that
+// completes the parent, and after a warp barrier the others, see every child's
+// records.  Returns how many of the parent's children have arrived.
 __device__ __forceinline__ int count_in(int par, int32_t *node_arrive) {
     int old;
-    asm volatile("atom.relaxed.gpu.global.add.s32 %0, [%1], 1;"
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;"
                  : "=r"(old)
                  : "l"(node_arrive + par)
                  : "memory");
@@ -625,13 +690,10 @@ __global__ void __launch_bounds__(256, NB_MOMENTS_MIN_CTAS) moments_kernel(
                 if (nodeQ) write_quad(id, q, nodeQ);
             }
         }
-        // internal nodes: the chunk's leaf records are device-visible before
-        // any lane counts a leaf in (the warp barrier, then the lane's fence).
-        // A climbing thread carries a member key (its leaf's first particle):
-        // every ancestor's cell follows from it and the ancestor's level, one
-        // up per step.
-        __syncwarp();
-        __threadfence();
+        // internal nodes.  A climbing lane carries a member key (its leaf's first
+        // particle): every ancestor's cell follows from it and the ancestor's
+        // level, one up per step.
+        __syncwarp();  // the chunk's leaf records, before any lane counts a leaf in
         int node = id0, par = -1, level = 0;
         uint64_t key = 0;
         if (leaf) {
@@ -640,25 +702,36 @@ __global__ void __launch_bounds__(256, NB_MOMENTS_MIN_CTAS) moments_kernel(
             key = key0;
         }
         for (;;) {
+            // each lane by itself while the parents it completes have few
+            // children (chains of single children below close particles)
             bool ready = false;
             int c0 = 0, nc = 0, up = -1;
-            if (par >= 0) {  // a root has none
+            while (par >= 0) {  // a root has none
                 if (par >= node) {  // parents precede their children
                     bad = true;
-                } else {
-                    // the parent's fields load beside the count-in atomic; the
-                    // lane that brings the last child has the parent computed
-                    c0 = node_link[par];
-                    nc = node_nchild[par];
-                    up = node_parent[par];
-                    ready = count_in(par, node_arrive) == nc;
+                    par = -1;
+                    break;
                 }
+                // the parent's fields load beside the count-in atomic; the
+                // lane that brings the last child has the parent computed
+                c0 = node_link[par];
+                nc = node_nchild[par];
+                up = node_parent[par];
+                if (count_in(par, node_arrive) != nc) {
+                    par = -1;
+                    break;
+                }
+                ready = nc > kAlone;
+                if (ready) break;
+                level--;
+                if (!internal_node_alone(L, par, c0, nc, level, key, refit, nn, box, G, node_count, nodeA,
+                                         nodeB, mass2, nodeQ))
+                    bad = true;  // still counted in above, so the counters stay consistent
+                node_arrive[par] = 0;
+                node = par;
+                par = up;
             }
-            // the completing lane's fence, then a warp barrier (ballots and
-            // shuffles order no memory): the team's lanes, which read the
-            // children, come after every child's count-in
-            if (ready) __threadfence();
-            __syncwarp();
+            __syncwarp();  // the teams' lanes come after every child's count-in
             unsigned rm = __ballot_sync(NB_FULL, ready);
             if (!rm) break;
             while (rm) {  // four parents at a time, eight lanes each
@@ -678,16 +751,12 @@ __global__ void __launch_bounds__(256, NB_MOMENTS_MIN_CTAS) moments_kernel(
                                     nodeA, nodeB, mass2, nodeQ))
                     bad = true;  // still counted in above, so the counters stay consistent
             }
-            // the teams' records are device-visible before any lane counts one in
-            __syncwarp();
-            __threadfence();
+            __syncwarp();  // the teams' records, before any lane counts one in
             if (ready) {
                 node_arrive[par] = 0;
                 node = par;
                 par = up;
                 level--;
-            } else {
-                par = -1;
             }
         }
     }

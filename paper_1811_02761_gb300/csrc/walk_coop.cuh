@@ -18,11 +18,10 @@
 //     walks every P-th of the child ranges found; the CTA that finishes last
 //     adds the P partial sums in part order.
 // It runs in two stages.  The first takes every group (where coop_walk, api.cu,
-// says so), or the
-// groups the one-warp walk cut at its quota; a part whose own list passes
-// a.cut_quota entries is cut again, its open ranges recorded.  The second stage
-// walks those records, again with P CTAs each, to the end: however uneven the
-// groups are, no CTA works much longer than the others.
+// says so), or the groups the one-warp walk cut at its quota; a part whose own
+// list passes a.cut_quota entries is cut again, its open ranges recorded.  The
+// second stage walks those records, again with P CTAs each, to the end: however
+// uneven the groups are, no CTA works much longer than the others.
 // The MAC is evaluated exactly as in the one-warp walk, so the list of every
 // group holds the same entries; only the order of the sums differs, and it
 // depends on the counts of groups and cuts alone, never on timing: which
