@@ -767,13 +767,18 @@ __global__ void __launch_bounds__(256, NB_MOMENTS_MIN_CTAS) moments_kernel(
 // one-lane teams above: same operations, same order), then the internal nodes
 // level by level from the deepest, with the records in shared memory (a tree
 // of up to kOneNodes nodes) and block barriers where the pass above has L2
-// round trips, a fence and an atomic count per level.  At n = 4096 (1023 nodes,
-// 13 levels) that pass takes 30 us, almost all of it the climb's chain, and
-// this one 23 us (warm caches), most of it the leaves' own chains and the code's
-// first fetch.
-constexpr int kMomentsOne = 8192;  // particles; leaves of at most 16 members
+// round trips and an atomic count per level.  For trees whose levels are one
+// round of the block's 128 teams: the internal nodes of a level are disjoint
+// and hold more than leaf_cap particles each.  Refit calls in us, the pass
+// above / this: 2000 particles, leaf_cap = 16, Plummer 69 / 60, on 64 points 94
+// / 82; leaf_cap = 1 120 / 95.  With more rounds it is the slower one: 8192
+// particles, leaf_cap = 1 130 / 221, 2000 on 1000 points 144 / 296.
+constexpr int kOneTeams = 128;
 constexpr int kOneNodes = 4096;
-__global__ void __launch_bounds__(1024) moments_one_kernel(
+static bool moments_one(int64_t n, int leaf_cap) {
+    return leaf_cap <= 16 && n / (leaf_cap + 1) <= kOneTeams;
+}
+__global__ void __launch_bounds__(8 * kOneTeams) moments_one_kernel(
     Layout L, int refit, const uint64_t *__restrict__ keys, const float4 *__restrict__ pos4,
     const SysBox *__restrict__ box, float G, DevState *ds, const int32_t *__restrict__ node_start,
     const int8_t *__restrict__ node_level, const int32_t *__restrict__ node_link,
@@ -911,10 +916,10 @@ void tree_moments(cudaStream_t s, const Layout &L, const uint64_t *keys, const f
                   const int32_t *node_link, int32_t *node_count, const int32_t *node_nchild,
                   int32_t *node_arrive, float4 *nodeA, float4 *nodeB, float2 *mass2,
                   float4 *nodeQ, int nsm, bool refit) {
-    if (L.n <= kMomentsOne && leaf_cap <= 16) {
+    if (moments_one(L.n, leaf_cap)) {
         const int smem = kOneNodes * (int)sizeof(NodeRec);
         cudaFuncSetAttribute(moments_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        moments_one_kernel<<<1, 1024, smem, s>>>(L, refit ? 1 : 0, keys, pos4, d_box, G, ds, node_start,
+        moments_one_kernel<<<1, 8 * kOneTeams, smem, s>>>(L, refit ? 1 : 0, keys, pos4, d_box, G, ds, node_start,
                                               node_level, node_link, node_count, node_nchild, nodeA,
                                               nodeB, mass2, nodeQ);
         return;
