@@ -1304,6 +1304,13 @@ static nbody_status step_impl(nbody_ctx *ctx, int32_t nsys, const int64_t *offse
     cudaStream_t s = ctx->stream;
     Layout L = make_layout(n, nsys);
     cudaError_t e = ensure_capacity(ctx, n, nsys, L.levels);
+    // The sorts swap the key and value buffers, and a call with an odd number of
+    // swaps left them the other way round for the next one, which then found
+    // another key and captured its step graph anew (3, 5, 7 steps of up to 8192
+    // particles, 4, 6, 8 of more).  Nothing of an earlier call is read from
+    // them here: every call starts with the lower address first.
+    if (e == cudaSuccess && ctx->keys.p > ctx->keys_alt.p) std::swap(ctx->keys, ctx->keys_alt);
+    if (e == cudaSuccess && ctx->vals.p > ctx->vals_alt.p) std::swap(ctx->vals, ctx->vals_alt);
     if (ctx->st_buf[0][0].bytes < (size_t)n * 8) ctx->growths++;
     for (int b = 0; b < 2 && e == cudaSuccess; b++) {
         for (int k = 0; k < 3 && e == cudaSuccess; k++) e = ensure(ctx->st_buf[b][k], (size_t)n * 8);
