@@ -12,6 +12,7 @@
 #include <string>
 #include <vector>
 
+#include "buffers.h"
 #include "internal.cuh"
 #include "scratch.h"
 
@@ -26,11 +27,6 @@ thread_local std::string g_last_error;
 void nb::set_stateless_error(const std::string &msg) { g_last_error = msg; }
 
 namespace {
-
-struct DevBuf {
-    void *p = nullptr;
-    size_t bytes = 0;
-};
 
 // What a captured step graph depends on: sizes, parameters and the buffers
 // its kernels were captured with.
@@ -170,24 +166,6 @@ bool is_device_ptr(const void *p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-cudaError_t ensure(DevBuf &b, size_t bytes) {
-    if (b.bytes >= bytes && b.p) return cudaSuccess;
-    if (b.p) {
-        cudaError_t e = cudaFree(b.p);
-        b.p = nullptr;
-        b.bytes = 0;
-        if (e != cudaSuccess) return e;
-    }
-    size_t want = bytes ? bytes : 16;
-    cudaError_t e = cudaMalloc(&b.p, want);
-    if (e != cudaSuccess) {
-        b.p = nullptr;
-        return e;
-    }
-    b.bytes = want;
-    return cudaSuccess;
-}
-
 template <typename T>
 T *P(DevBuf &b) {
     return reinterpret_cast<T *>(b.p);
@@ -308,49 +286,51 @@ int64_t node_capacity(int64_t n, int levels, int leaf_cap, int nsys) {
 }
 
 cudaError_t ensure_capacity(nbody_ctx *c, int64_t n, int nsys, int levels) {
-    cudaError_t e;
-#define NB_E(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
+    cudaError_t e = cudaSuccess;
+    const size_t m = (size_t)n;
     if (n > c->cap_n) {
         c->growths++;
-        NB_E(ensure(c->keys, n * 8)); NB_E(ensure(c->keys_alt, n * 8));
-        NB_E(ensure(c->vals, n * 4)); NB_E(ensure(c->vals_alt, n * 4));
-        NB_E(ensure(c->pos4, n * 16)); NB_E(ensure(c->delta, n + 1)); NB_E(ensure(c->leaflev, n));
-        NB_E(ensure(c->rs_temp, std::max(radix_temp_bytes(n), nosort_temp_bytes(n))));
-        NB_E(ensure(c->tree_temp, tree_temp_bytes(n, kMaxLevels)));
-        NB_E(ensure(c->grp_temp, (size_t)((n + 4095) / 4096 + 64) * 4));
-        NB_E(ensure(c->gflag, (n + 15) / 16 * 16));
-        NB_E(cudaMemsetAsync(c->gflag.p, 0, c->gflag.bytes, c->stream));  // every build leaves it zero
-        NB_E(ensure(c->grp_first, n * 4)); NB_E(ensure(c->grp_count, n * 4));
-        NB_E(ensure(c->grp_sphere, n * 16)); NB_E(ensure(c->grp_sys, n * 4));
-        NB_E(ensure(c->grp_alpha, n * 4)); NB_E(ensure(c->grp_cost, n * 4));
-        NB_E(ensure(c->grp_order, n * 4));
-        NB_E(ensure(c->acc_s, n * 16)); NB_E(ensure(c->aold_s, n * 4));
-        c->cap_n = n;
+        e = grow(c->cap_n, n,
+                 {{&c->keys, m * 8}, {&c->keys_alt, m * 8}, {&c->vals, m * 4}, {&c->vals_alt, m * 4},
+                  {&c->pos4, m * 16}, {&c->delta, m + 1}, {&c->leaflev, m},
+                  {&c->rs_temp, std::max(radix_temp_bytes(n), nosort_temp_bytes(n))},
+                  {&c->tree_temp, tree_temp_bytes(n, kMaxLevels)},
+                  {&c->grp_temp, ((m + 4095) / 4096 + 64) * 4}, {&c->gflag, (m + 15) / 16 * 16},
+                  {&c->grp_first, m * 4}, {&c->grp_count, m * 4}, {&c->grp_sphere, m * 16},
+                  {&c->grp_sys, m * 4}, {&c->grp_alpha, m * 4}, {&c->grp_cost, m * 4},
+                  {&c->grp_order, m * 4}, {&c->acc_s, m * 16}, {&c->aold_s, m * 4}});
+        // every build leaves the flags zero
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->gflag.p, 0, c->gflag.bytes, c->stream);
+        if (e != cudaSuccess) {
+            c->cap_n = 0;
+            return e;
+        }
     }
-    int64_t cn = node_capacity(n, levels, c->cfg.leaf_cap, nsys);
+    const int64_t cn = node_capacity(n, levels, c->cfg.leaf_cap, nsys);
     if (cn > c->cap_nodes) {
+        const size_t k = (size_t)cn;
         c->growths++;
-        NB_E(ensure(c->node_start, cn * 4)); NB_E(ensure(c->node_level, cn));
-        NB_E(ensure(c->node_parent, cn * 4)); NB_E(ensure(c->node_link, cn * 4));
-        NB_E(ensure(c->node_count, cn * 4)); NB_E(ensure(c->node_nchild, cn * 4));
-        NB_E(ensure(c->node_arrive, cn * 4));
-        NB_E(ensure(c->nodeA, cn * 16)); NB_E(ensure(c->nodeB, cn * 16));
-        NB_E(ensure(c->mass2, cn * 8)); NB_E(ensure(c->nodeQ, cn * 32));
-        c->cap_nodes = cn;
+        e = grow(c->cap_nodes, cn,
+                 {{&c->node_start, k * 4}, {&c->node_level, k}, {&c->node_parent, k * 4},
+                  {&c->node_link, k * 4}, {&c->node_count, k * 4}, {&c->node_nchild, k * 4},
+                  {&c->node_arrive, k * 4}, {&c->nodeA, k * 16}, {&c->nodeB, k * 16},
+                  {&c->mass2, k * 8}, {&c->nodeQ, k * 32}});
+        if (e != cudaSuccess) return e;
     }
     if (nsys > c->cap_sys) {
+        const size_t k = (size_t)nsys;
         c->growths++;
-        NB_E(ensure(c->sys_off, (size_t)(nsys + 1) * 8)); NB_E(ensure(c->sys_box, (size_t)nsys * sizeof(SysBox)));
-        NB_E(ensure(c->sys_boxord, (size_t)nsys * 24 + 4)); NB_E(ensure(c->sys_eps2, (size_t)nsys * 4));
-        NB_E(ensure(c->sys_eps, (size_t)nsys * 4));
-        NB_E(ensure(c->sys_root, (size_t)nsys * 4));
-        c->cap_sys = nsys;
+        e = grow(c->cap_sys, nsys,
+                 {{&c->sys_off, (k + 1) * 8}, {&c->sys_box, k * sizeof(SysBox)},
+                  {&c->sys_boxord, k * 24 + 4}, {&c->sys_eps2, k * 4}, {&c->sys_eps, k * 4},
+                  {&c->sys_root, k * 4}});
+        if (e != cudaSuccess) return e;
         // empty extents and a zero count of blocks: every build leaves them so
         launch_bbox_init(c->stream, nsys, P<uint32_t>(c->sys_boxord));
-        NB_E(cudaMemsetAsync(P<uint32_t>(c->sys_boxord) + (size_t)nsys * 6, 0, 4, c->stream));
+        e = cudaMemsetAsync(P<uint32_t>(c->sys_boxord) + k * 6, 0, 4, c->stream);
+        if (e != cudaSuccess) c->cap_sys = 0;
     }
-#undef NB_E
-    return cudaSuccess;
+    return e;
 }
 
 Layout make_layout(int64_t n, int nsys) {
