@@ -794,7 +794,7 @@ nbody_status compute_order(nbody_ctx *c, const float *pcost, const int32_t **ord
     if (sched == NBODY_SCHED_MLP) {
         launch_features(c);
         const float *nrm = c->mlp_norm_set ? P<float>(c->mlp_norm) : nullptr;
-        launch_mlp_forward(c->stream, png, 0, P<float>(c->feat),
+        launch_mlp_forward(c->stream, png, P<float>(c->feat),
                            reinterpret_cast<const __nv_bfloat16 *>(c->mlp_wb.p), nrm,
                            nrm ? nrm + 16 : nullptr, P<float>(c->score), c->nsm);
     } else {
@@ -1936,7 +1936,7 @@ nbody_status nbody_mlp_predict(nbody_ctx *ctx, float *pred, float *features, int
     if (ensure_mlp_buffers(ctx) != cudaSuccess) return fail(ctx, NBODY_ENOMEM, "allocation");
     launch_features(ctx);
     const float *nrm = ctx->mlp_norm_set ? P<float>(ctx->mlp_norm) : nullptr;
-    launch_mlp_forward(ctx->stream, &ctx->ds->ngroups, 0, P<float>(ctx->feat),
+    launch_mlp_forward(ctx->stream, &ctx->ds->ngroups, P<float>(ctx->feat),
                        reinterpret_cast<const __nv_bfloat16 *>(ctx->mlp_wb.p), nrm,
                        nrm ? nrm + 16 : nullptr, P<float>(ctx->score), ctx->nsm);
     NB_CUDA(ctx, cudaGetLastError());

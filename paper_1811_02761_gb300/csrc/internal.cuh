@@ -193,8 +193,7 @@ void nosort(cudaStream_t s, uint64_t *keys, uint64_t *kout, uint32_t *vscr, uint
 void nosort_hint_gather(cudaStream_t s, int64_t n, const uint64_t *keys, const uint32_t *hint,
                         uint64_t *kout, uint32_t *vout);
 int nosort_kernels();
-// The stable sort of up to kRankSortMax keys below 2^63 in any order, in one
-// launch: kout the sorted keys, vout the input index of each.
+// The stable sort of up to kRankSortMax keys in any order, in one launch: kout the sorted keys, vout the input index of each.
 constexpr int kRankSortMax = 8192;
 cudaError_t rank_sort(cudaStream_t s, const uint64_t *keys, int64_t n, uint64_t *kout, uint32_t *vout);
 // True for memory the current device dev can read in place (its own device
@@ -355,7 +354,7 @@ void launch_mlp_features(cudaStream_t s, const Layout &L, const DevState *ds,
                          const float4 *grp_sphere, const int32_t *grp_sys, const float *aold,
                          const uint64_t *keys, const float4 *nodeA, const int32_t *sys_root,
                          const SysBox *box, const int64_t *off, float *feat, int nsm);
-void launch_mlp_forward(cudaStream_t s, const int32_t *pn, int64_t n, const float *feat,
+void launch_mlp_forward(cudaStream_t s, const int32_t *pn, const float *feat,
                         const __nv_bfloat16 *wb, const float *norm, const float *tnorm,
                         float *pred, int nsm);
 // gpart: kMlpParams floats and lpart: one per block of kMlpGradBlock samples.

@@ -168,7 +168,7 @@ __device__ __forceinline__ float mlp_fwd(const MlpSmem &S, const float *x, float
 
 // tnorm (nullable): target mean and standard deviation; the network output
 // is de-standardised with them.
-__global__ void __launch_bounds__(128) mlp_forward_kernel(const int32_t *__restrict__ pn, int64_t n_host,
+__global__ void __launch_bounds__(128) mlp_forward_kernel(const int32_t *__restrict__ pn,
                                                           const float *__restrict__ feat,
                                                           const __nv_bfloat16 *__restrict__ wb,
                                                           const float *__restrict__ norm,
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(128) mlp_forward_kernel(const int32_t *__restr
     __shared__ float xr[128][kIn + 1];
     load_weights(S, wb, nullptr, norm);
     const float tm = tnorm ? tnorm[0] : 0.0f, ts = tnorm ? tnorm[1] : 1.0f;
-    const int64_t n = pn ? (int64_t)*pn : n_host;
+    const int64_t n = *pn;
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n;
          g += (int64_t)gridDim.x * blockDim.x) {
         float h2[kH];
@@ -467,10 +467,10 @@ void launch_mlp_features(cudaStream_t s, const Layout &L, const DevState *ds,
                                                 aold, keys, nodeA, sys_root, box, off, feat);
 }
 
-void launch_mlp_forward(cudaStream_t s, const int32_t *pn, int64_t n, const float *feat,
+void launch_mlp_forward(cudaStream_t s, const int32_t *pn, const float *feat,
                         const __nv_bfloat16 *wb, const float *norm, const float *tnorm,
                         float *pred, int nsm) {
-    mlp_forward_kernel<<<nsm * 4, 128, 0, s>>>(pn, n, feat, wb, norm, tnorm, pred);
+    mlp_forward_kernel<<<nsm * 4, 128, 0, s>>>(pn, feat, wb, norm, tnorm, pred);
 }
 
 cudaError_t launch_mlp_train_step(cudaStream_t s, const float *feat, const float *target,

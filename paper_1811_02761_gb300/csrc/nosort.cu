@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(32 * RK_WARPS) rank_sort_kernel(const uint64_t
     const uint64_t ki = i < n ? rk_keys[i] : 0ull;
     const int per = (n + RK_WARPS - 1) / RK_WARPS;
     const int j0 = min(n, w * per), j1 = min(n, j0 + per);
-    // keys are below 2^63: an equal key counts when its index is smaller
+    // an equal key counts when its index is smaller
     const int mid = min(max(i, j0), j1);
     int c = 0;
 #pragma unroll 8

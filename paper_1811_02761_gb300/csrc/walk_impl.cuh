@@ -471,7 +471,10 @@ __device__ __forceinline__ bool over_quota(const WalkArgs &a, int entries, int n
 // spilled up to 1.3 KB at 80 registers, and 16 warps per SM without spills beat
 // 24 with them (galaxy 300007, quadrupoles, 2^-12: 1.60 -> 1.53 ms, 96
 // registers 1.52; Plummer 4096 with quadrupoles, cooperative, 67 -> 57 us;
-// compensated, 300000 at 2^-20, 9.5 -> 9.1 ms).
+// compensated, 300000 at 2^-20, 9.5 -> 9.1 ms).  The cooperative instances with
+// plain monopole sums at three slots still spill 76 to 102 bytes at 80; with 96,
+// and so two CTAs per SM instead of three, they were slower (Plummer 4096 38 ->
+// 53 us).
 #ifndef NB_WALK_REGS_2
 #define NB_WALK_REGS_2 64
 #endif
