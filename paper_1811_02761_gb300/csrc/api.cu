@@ -483,16 +483,18 @@ nbody_status upload_systems(nbody_ctx *c, int nsys, const int64_t *offsets, cons
     int64_t *off = reinterpret_cast<int64_t *>(c->h_sys);
     float *e1 = reinterpret_cast<float *>(c->h_sys + ob), *e2 = e1 + nsys;
     std::memcpy(off, offsets, ob);
-    c->sys_max = 0;
-    c->sys_mean = 0.0;
+    const float eps = c->cfg.eps;
+    int64_t largest = 0, squares = 0;  // of at most n^2 < 2^62 in all
     for (int s = 0; s < nsys; s++) {
-        const float e = eps_sys ? eps_sys[s] : c->cfg.eps;
+        const float e = eps_sys ? eps_sys[s] : eps;
         e1[s] = e;
         e2[s] = e * e;
         const int64_t ns = offsets[s + 1] - offsets[s];
-        c->sys_max = std::max(c->sys_max, ns);
-        c->sys_mean += (double)ns * (double)ns / (double)std::max<int64_t>(offsets[nsys], 1);
+        largest = std::max(largest, ns);
+        squares += ns * ns;
     }
+    c->sys_max = largest;
+    c->sys_mean = (double)squares / (double)std::max<int64_t>(offsets[nsys], 1);
     NB_CUDA(c, cudaMemcpyAsync(c->sys_off.p, off, ob, cudaMemcpyHostToDevice, c->stream));
     NB_CUDA(c, cudaMemcpyAsync(c->sys_eps2.p, e2, eb, cudaMemcpyHostToDevice, c->stream));
     NB_CUDA(c, cudaMemcpyAsync(c->sys_eps.p, e1, eb, cudaMemcpyHostToDevice, c->stream));
