@@ -510,6 +510,9 @@ __global__ void __maxnreg__((walk_regs<IPL, QUAD || COMP>())) walk_kernel(WalkAr
     const int ng = a.nactive ? *a.nactive : ds->ngroups;
     const int nnodes = ds->nnodes;
     const int npart = (int)a.n;
+    // without this test the compiler's schedule of the loop is 1 % slower (walk
+    // at N = 2^23 6.175 ms, 6.112 with it; a forest of 512 systems 11.27, 11.13)
+    if (ng <= 0) return;
     const unsigned lt = lanemask_lt();
     int max_sp = 0;
     unsigned long long warp_entries = 0, warp_inter = 0, warp_quad = 0;
