@@ -122,8 +122,10 @@ typedef struct {
                             from dt_i = sqrt(2 block_eta eps / |a_i|) (the paper's
                             code uses block steps, Sect. 1; this criterion is
                             a reading); only groups with a particle whose step
-                            ends at a tick are walked.  nsteps counts steps of
-                            dt; the state returned is synchronised.  Not with
+                            ends at a tick are walked.  Walks and steps of such
+                            a context sum every group's list in one fixed order
+                            (not with block_eta > 1, which asks for one level).
+                            nsteps counts steps of dt; the state returned is synchronised.  Not with
                             use_graph; the stream is synchronised after every
                             processed tick.                                 */
     float block_eta;     /* accuracy parameter of the block step criterion

@@ -594,6 +594,12 @@ double ordinary_list(const nbody_ctx *c, bool geometric) {
                                : std::pow(std::max(c->cfg.delta_acc, 1e-12f) * 512.0, -0.485));
 }
 
+// Contexts that are walked in one fixed order throughout (walk_ordered.cuh):
+// those with block steps, their forces between steps included.  A block_eta
+// above 1 (steps longer than a free fall through the softening) is no accuracy
+// criterion but asks for one level: shared steps, walked as those are.
+bool ordered_run(const nbody_config &c) { return c.block_levels > 0 && c.block_eta <= 1.0f; }
+
 // Which walk: the cooperative one for all groups, or one warp per group with
 // the cooperative one for the groups cut at the quota.  (Block steps:
 // walk_ordered.cuh.)  One warp per group takes as long as the longest list's
@@ -820,7 +826,7 @@ nbody_status compute_order(nbody_ctx *c, const float *pcost, const int32_t **ord
 
 // Walk over the current groups; aold_s (sorted) must hold |a_old|, unless the
 // group pass has formed alpha and reset the queues already (prepared).
-// ordered (not with geometric or phi): the ordered walk.
+// ordered: the ordered walk.
 nbody_status run_walk(nbody_ctx *c, bool geometric, bool phi, bool safe, const int32_t *perm,
                       float *ax, float *ay, float *az, float *ph, float4 *acc_sorted,
                       bool reset_accumulators = true, const float *pcost = nullptr,
@@ -1076,7 +1082,7 @@ nbody_status nbody_walk(nbody_ctx *ctx, const float *a_old, float *ax, float *ay
     } else {
         // bootstrap: geometric criterion first, its |a| feeds Eq. 2
         st = run_walk(ctx, true, false, safe, nullptr, nullptr, nullptr, nullptr, nullptr,
-                      P<float4>(ctx->acc_s));
+                      P<float4>(ctx->acc_s), true, nullptr, nullptr, nullptr, false, ordered_run(ctx->cfg));
         if (st != NBODY_OK) return st;
         launch_acc_mag(s, n, P<float4>(ctx->acc_s), P<float>(ctx->aold_s));
         ctx->kernels += 1;
@@ -1084,7 +1090,8 @@ nbody_status nbody_walk(nbody_ctx *ctx, const float *a_old, float *ax, float *ay
     const bool have_pcost = ctx->costs_valid && ctx->pcost_walk.p;
     st = run_walk(ctx, false, want_phi, safe, (const int32_t *)P<uint32_t>(ctx->vals),
                   (float *)dax, (float *)day, (float *)daz, (float *)dph, nullptr, true,
-                  have_pcost ? P<float>(ctx->pcost_walk) : nullptr);
+                  have_pcost ? P<float>(ctx->pcost_walk) : nullptr, nullptr, nullptr, false,
+                  ordered_run(ctx->cfg));
     if (st != NBODY_OK) return st;
     if (ensure(ctx->pcost_walk, (size_t)n * 4) == cudaSuccess) {
         launch_spread_cost(s, &ctx->ds->ngroups, P<int32_t>(ctx->grp_first), P<int32_t>(ctx->grp_count),
@@ -1250,10 +1257,9 @@ static nbody_status block_steps(nbody_ctx *ctx, const Layout &L, StepState *S, i
         launch_block_active_groups(q, ctx->ds, P<int32_t>(ctx->grp_first), P<int32_t>(ctx->grp_count),
                                    S[cur].lvl, T, K, P<int32_t>(ctx->grp_order), dact, ctx->nsm);
         ctx->kernels += 1;
-        // particles on several levels: the ordered walk.  All on level 0: these
-        // are shared steps, and walked as those are
         st = run_walk(ctx, false, false, safe, nullptr, nullptr, nullptr, nullptr, nullptr, acc,
-                      false, nullptr, P<int32_t>(ctx->grp_order), dact, true, kmax > 0);
+                      false, nullptr, P<int32_t>(ctx->grp_order), dact, true,
+                      kmax > 0 || ordered_run(ctx->cfg));
         if (st != NBODY_OK) return st;
         NB_CUDA(ctx, pool_event(ctx, &e2));
         NB_CUDA(ctx, cudaEventRecord(e2, q));

@@ -335,7 +335,7 @@ struct WalkShape {
     bool quad;                  // accepted nodes add their quadrupole
     int warps_per_block;
     bool coop_only;             // the cooperative kernel alone (WalkArgs::coop_all)
-    bool ordered;               // the ordered walk alone (no potential, |a_old| given)
+    bool ordered;               // the ordered walk alone (runs with block steps)
     int *warps_launched;        // host, nullable: receives the resident walk warps
 };
 // The walk of one warp per group (not with sh.coop_only), then the

@@ -1,14 +1,15 @@
-// walk_ordered.cuh -- the tree walk of the block time steps: one warp per
+// walk_ordered.cuh -- the tree walk of runs with block time steps: one warp per
 // group from the root to the end, in one order of operations.
 //
 // The steps of a block step are long (dt itself on level 0), so the FP32
 // rounding of the accelerations reaches the FP64 positions through the FP32
 // velocities: Plummer spheres of 2,000 to 100,000 particles at dt = 1/8, walked
 // in this order and cooperatively, part by 5e-10 of the positions (2-norm) in
-// one call and by 1.5e-9 in two.  A run followed with block steps is therefore
-// walked in an order that depends on the group alone -- not on how many groups
-// are active, nor on quotas and parts: the list is filled round by round
-// (accepted nodes, then the particles of opened leaves, 32 at a time) and
+// one call and by 1.5e-9 in two, and a level decision that falls the other way
+// by up to 4e-7.  A run followed with block steps is therefore walked, from its
+// first forces on, in an order that depends on the group alone -- not on how
+// many groups are active, nor on quotas and parts: the list is filled round by
+// round (accepted nodes, then the particles of opened leaves, 32 at a time) and
 // flushed when the next append would not fit, and an interaction is
 // (m / r) / r / r.
 //
@@ -21,9 +22,8 @@
 
 namespace nb {
 
-template <int IPL, bool COMP, bool SAFE, bool QUAD>
-__global__ void __maxnreg__((walk_regs<IPL, QUAD || COMP>())) ordered_walk_kernel(WalkArgs a) {
-    constexpr bool PHI = false;
+template <int IPL, bool PHI, bool COMP, bool SAFE, bool QUAD>
+__global__ void __maxnreg__((walk_regs<IPL, QUAD || COMP>())) ordered_walk_kernel(WalkArgs a, int geometric) {
     extern __shared__ __align__(16) unsigned char walk_smem[];
     const int D = a.list_depth, S = a.stack_depth;
     const int DQ = QUAD ? walk_quad_depth(D) : 0;
@@ -51,7 +51,7 @@ __global__ void __maxnreg__((walk_regs<IPL, QUAD || COMP>())) ordered_walk_kerne
         const int g = a.order ? a.order[qi] : qi;
         const int first = a.grp_first[g], cnt = a.grp_count[g];
         const float4 sph = a.grp_sphere[g];
-        const float alpha = a.grp_alpha[g];
+        const float alpha = geometric ? 0.0f : a.grp_alpha[g];
         const int sys = a.grp_sys[g];
         const float eps2 = a.sys_eps2[sys];
 
@@ -95,8 +95,13 @@ __global__ void __maxnreg__((walk_regs<IPL, QUAD || COMP>())) ordered_walk_kerne
             const float4 A = __ldg(&a.nodeA[nd]), B = __ldg(&a.nodeB[nd]);
             const float dx = A.x - sph.x, dy = A.y - sph.y, dz = A.z - sph.z;
             const float d = sqrt_fast(fmaf(dz, dz, fmaf(dy, dy, dx * dx))) - sph.w;
-            const float d2 = d * d;
-            const bool accept = has && d > B.x && B.y <= alpha * (d2 * d2);
+            bool accept;
+            if (geometric) {
+                accept = has && d > B.x && B.x <= a.theta * d;
+            } else {
+                const float d2 = d * d;
+                accept = has && d > B.x && B.y <= alpha * (d2 * d2);
+            }
             const int link = __float_as_int(B.z), meta = __float_as_int(B.w);
             const bool leaf = (meta & 1) != 0;
             const int mcount = meta >> 1;
@@ -173,8 +178,9 @@ __global__ void __maxnreg__((walk_regs<IPL, QUAD || COMP>())) ordered_walk_kerne
         }
         __syncwarp();
 
+        const float self = SAFE ? 0.0f : rsqrt_fast(eps2);
         group_sums<IPL, PHI, COMP>(tile, cnt, I, [&](int idx, const float (&r)[4], float mi) {
-            store_force<PHI>(a, first + idx, r, mi, a.G, 0.0f);
+            store_force<PHI>(a, first + idx, r, mi, a.G, self);
         });
         entries += qentries;
         if (lane == 0 && a.grp_cost) a.grp_cost[g] = entries;
@@ -199,9 +205,14 @@ cudaError_t launch_ordered_ipl(cudaStream_t s, const WalkArgs &a, const WalkShap
     const int threads = 32 * sh.warps_per_block;
     const size_t smem =
         (size_t)sh.warps_per_block * walk_smem_per_warp(a.list_depth, a.stack_depth, QUAD);
-    void (*k)(WalkArgs);
-    if (sh.compensated) k = sh.safe ? ordered_walk_kernel<IPL, true, true, QUAD> : ordered_walk_kernel<IPL, true, false, QUAD>;
-    else k = sh.safe ? ordered_walk_kernel<IPL, false, true, QUAD> : ordered_walk_kernel<IPL, false, false, QUAD>;
+    void (*k)(WalkArgs, int);
+    if (sh.potential) {
+        if (sh.compensated) k = sh.safe ? ordered_walk_kernel<IPL, true, true, true, QUAD> : ordered_walk_kernel<IPL, true, true, false, QUAD>;
+        else k = sh.safe ? ordered_walk_kernel<IPL, true, false, true, QUAD> : ordered_walk_kernel<IPL, true, false, false, QUAD>;
+    } else {
+        if (sh.compensated) k = sh.safe ? ordered_walk_kernel<IPL, false, true, true, QUAD> : ordered_walk_kernel<IPL, false, true, false, QUAD>;
+        else k = sh.safe ? ordered_walk_kernel<IPL, false, false, true, QUAD> : ordered_walk_kernel<IPL, false, false, false, QUAD>;
+    }
     cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     int per_sm = 0;
@@ -209,7 +220,7 @@ cudaError_t launch_ordered_ipl(cudaStream_t s, const WalkArgs &a, const WalkShap
     if (err != cudaSuccess) return err;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     if (sh.warps_launched) *sh.warps_launched = nsm * per_sm * sh.warps_per_block;
-    k<<<nsm * per_sm, threads, smem, s>>>(a);
+    k<<<nsm * per_sm, threads, smem, s>>>(a, sh.geometric ? 1 : 0);
     return cudaGetLastError();
 }
 

@@ -54,3 +54,35 @@ CASES = [
 @pytest.mark.parametrize("n,seed,config,recorded", CASES)
 def test_positions_after_two_calls(n, seed, config, recorded):
     assert hashlib.sha256(positions(n, seed, **config).tobytes()).hexdigest()[:16] == recorded
+
+
+def run_from_first_forces(n, seed, **config):
+    """Forces and potential without |a_old|, then one call of block steps."""
+    x, v, _ = state(n, seed)
+    dev = lambda t: [torch.from_numpy(np.ascontiguousarray(c)).cuda() for c in t]  # noqa: E731
+    X, V = dev(x), dev(v)
+    M = torch.full((n,), 1.0 / n, device="cuda", dtype=torch.float32)
+    A = [torch.empty(n, device="cuda", dtype=torch.float32) for _ in range(4)]
+    ctx = nb.nbody_create(nb.nbody_config_default(eps=1.0 / 64, block_levels=6, want_potential=1, **config))
+    try:
+        nb.nbody_build(ctx, *[t.float() for t in X], M)
+        nb.nbody_walk(ctx, None, *A)
+        first = torch.stack(A).cpu().numpy()
+        nb.nbody_step(ctx, *X, *V, M, *A[:3], 1.0 / 8, 1)
+    finally:
+        nb.nbody_destroy(ctx)
+    return np.concatenate([first.ravel().view(np.uint8), np.stack([t.cpu().numpy() for t in X]).ravel().view(np.uint8)])
+
+
+FIRST = [
+    (2000, 6, {}, "3bb0e24b4aa66e39"),
+    (9001, 7, dict(compensated=1, rebuild_interval=4), "45c6109f2b555608"),
+    (30011, 8, dict(quadrupole=1), "8b9f14fab04d2c16"),
+    (150001, 9, dict(group_size=48), "89ff0105e60c8085"),
+]
+
+
+@pytest.mark.parametrize("n,seed,config,recorded", FIRST)
+def test_run_from_its_first_forces(n, seed, config, recorded):
+    got = run_from_first_forces(n, seed, **config)
+    assert hashlib.sha256(got.tobytes()).hexdigest()[:16] == recorded
