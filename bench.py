@@ -48,9 +48,9 @@ FP32_LANES_PER_SM = 128
 # warm-up-step walk, per particle; at another N the launch is scaled by
 # particles.  It is reported only while the walk source is the one the
 # counters were taken on (sha256 of walk_impl.cuh).
-WALK_TRAFFIC = {"bytes_per_particle": (230.606e6 + 110.991e6) / 8388608,
+WALK_TRAFFIC = {"bytes_per_particle": (230.856e6 + 111.131e6) / 8388608,
                 "n_captured": 8388608,
-                "walk_impl_sha256": "fb4f6dabbe23e1048edea65aeb64b61204e5fa5d06dd3ebbe89c8a98bba97f80",
+                "walk_impl_sha256": "b0264fb6b419e120ccf41bf1aeaeaa432b446c756b169604cac5f25a354bc2e3",
                 "capture": "profiles/walk_kernel_traffic_galaxy_2e23.md"}
 
 

@@ -160,8 +160,8 @@ typedef struct {
     int64_t quad_interactions; /* of `interactions`, those with quadrupole
                               nodes (quadrupole = 1)                          */
     int32_t walk_warps;    /* resident walk warps of the last walk launch (one
-                              warp per group; for small systems, whose groups
-                              are walked by whole CTAs, those CTAs' warps)     */
+                              warp per group; where all groups are walked by
+                              whole CTAs, those CTAs' warps)                   */
 } nbody_stats;
 
 typedef struct nbody_ctx nbody_ctx;
