@@ -94,7 +94,10 @@ struct nbody_ctx {
     char *h_sys = nullptr;     // pinned: offsets, eps, eps^2 on their way to the device
     size_t h_sys_bytes = 0;
     int64_t sys_max = 0;   // particles of the largest system of the last build or step
-    double sys_mean = 0;   // and of the system that a particle is in, on average
+    struct SizeBin {       // its systems by the power of two of their size
+        int64_t particles = 0, systems = 0;
+    } sys_bin[32];
+    double sys_mean = 0;   // particles of the system that a particle is in, on average
     cudaEvent_t sys_ev = nullptr;
 
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
@@ -461,6 +464,10 @@ nbody_status refit_tree_groups(nbody_ctx *c, const Layout &L, const float *aold 
     return NBODY_OK;
 }
 
+// Up to this many systems their sizes are binned for the choice of the walk (a
+// few ns of host time each); with more, all count as of the mean size.
+constexpr int kBinnedSystems = 4096;
+
 // Upload the CSR offsets, per-system eps and eps^2, from page-locked memory:
 // the copies are ordered before the call's kernels and need no wait (from
 // pageable memory they cost three staged copies and a synchronisation, about
@@ -495,6 +502,16 @@ nbody_status upload_systems(nbody_ctx *c, int nsys, const int64_t *offsets, cons
     }
     c->sys_max = largest;
     c->sys_mean = (double)squares / (double)std::max<int64_t>(offsets[nsys], 1);
+    for (auto &b : c->sys_bin) b = {};
+    if (nsys <= kBinnedSystems) {
+        for (int s = 0; s < nsys; s++) {
+            const int64_t ns = offsets[s + 1] - offsets[s];
+            if (ns < 1) continue;
+            auto &b = c->sys_bin[63 - __builtin_clzll((unsigned long long)ns)];
+            b.particles += ns;
+            b.systems++;
+        }
+    }
     NB_CUDA(c, cudaMemcpyAsync(c->sys_off.p, off, ob, cudaMemcpyHostToDevice, c->stream));
     NB_CUDA(c, cudaMemcpyAsync(c->sys_eps2.p, e2, eb, cudaMemcpyHostToDevice, c->stream));
     NB_CUDA(c, cudaMemcpyAsync(c->sys_eps.p, e1, eb, cudaMemcpyHostToDevice, c->stream));
@@ -603,24 +620,30 @@ bool ordered_run(const nbody_config &c) { return c.block_levels > 0 && c.block_e
 // Which walk: the cooperative one for all groups, or one warp per group with
 // the cooperative one for the groups cut at the quota.  (Block steps:
 // walk_ordered.cuh.)  One warp per group takes as long as the longest list's
-// chain, a launch and 0.05 + 0.0014 G us per entry, as long as most warps have
+// chain, a launch and 0.03 + 0.0014 G us per entry, as long as most warps have
 // one group; the cooperative walk a launch (more with quadrupoles or
 // compensated sums) and a time per group that grows with its list.  Lists are
 // estimated by ordinary_list and the particles of a system, the groups as
-// 0.7 G particles each and at least one per system.  Fitted to 1040 walks of
-// 2 to 200003 particles, 1 to 16000 systems, groups of 16 to 96, quadrupoles,
-// compensated sums and delta_acc = 2^-14 to 2^-5: within 3 % of the better one
-// of the two (geometric mean; a line by particles alone, 2^17, was 28 %
-// off).  Both sides in us, one warp / cooperative: galaxy, G = 64, N = 4096
-// 187 / 41, 100003 252 / 201, 200003 318 / 350; N = 100003, G = 16 146 / 396; 12000
-// systems of 10 particles 34 / 181; 256 particles, compensated, 25 / 42.
+// 0.7 G particles each and at least one per system.  Fitted to 1903 walks of
+// 2 to 300000 particles, 1 to 16000 systems of equal and of very different
+// sizes, groups of 16 to 128, quadrupoles, compensated sums and delta_acc =
+// 2^-20 to 2^-5: within 3 % of the better one of the two (geometric mean; a line
+// by particles alone, 2^17, was 23 % off).  Both sides in us, one warp /
+// cooperative: galaxy, G = 64, N = 4096 187 / 41, 100003 252 / 201, 200003 318 /
+// 350; N = 100003, G = 16 146 / 396; 12000 systems of 10 particles 34 / 181; 256
+// particles, compensated, 25 / 42; 1500 systems of 1 to 1266 particles 109 / 235.
 bool coop_walk(const nbody_ctx *c, bool geometric) {
     const double G = c->cfg.group_size, ordinary = ordinary_list(c, geometric);
-    const double groups = c->L.n / (0.7 * G) + c->L.nsys;
     const bool more = c->cfg.quadrupole != 0 || use_compensation(c->cfg);
-    const double chain = 5.0 + std::min((double)c->sys_max, ordinary) * (0.05 + 0.0014 * G);
-    const double coop = (more ? 70.0 : 30.0) +
-                        groups * (0.002 + std::min(c->sys_mean, ordinary) * (2.5e-5 + 2e-7 * G));
+    const double chain = 5.0 + std::min((double)c->sys_max, ordinary) * (0.03 + 0.0014 * G);
+    double coop = more ? 82.0 : 32.0;
+    auto add = [&](double particles, double systems, double size) {
+        coop += (particles / (0.7 * G) + systems) * (0.008 + std::min(size, ordinary) * (1.5e-5 + 1e-7 * G));
+    };
+    if (c->L.nsys > kBinnedSystems) add((double)c->L.n, c->L.nsys, c->sys_mean);
+    else
+        for (const auto &b : c->sys_bin)
+            if (b.systems) add((double)b.particles, (double)b.systems, (double)b.particles / (double)b.systems);
     return coop < chain;
 }
 
